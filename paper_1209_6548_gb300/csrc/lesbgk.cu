@@ -1094,14 +1094,48 @@ namespace {
 
 int pick_launch(lesbgk *h) {
   const int nx = h->p.nx, ny = h->p.ny;
-  // one node per lane, 28 nodes per strip (two halo lanes per side); default
-  // segments of 32 rows (D2Q16, D3Q64) or 128 rows (D2Q36): measured best on
-  // the 4096^2 periodic case (D2Q36: 961 us per step at 128 rows, 988 us at
-  // 32, where the three prologue rows per segment weigh more)
+  // One node per lane, 28 nodes per strip (two halo lanes per side).  Rows per
+  // segment: a segment costs its rows plus a prologue (the stencil rows and
+  // the ring's first loads, about kPro rows' time); a row takes one warp's
+  // latency or, with k blocks on the SM, k times a block's `share` of the
+  // issue slots, whichever is more (one-block against full-chip runs, in units
+  // of that latency); past one wave the blocks' ends are spread over half a
+  // segment.  Small grids so get short segments, middle ones the longest that
+  // fill every SM evenly (us per step with 32 or, D2Q36 and D3Q216, 128 rows ->
+  // now; 4x64 D2Q16 20.5 -> 4.1, D2Q36 69.7 -> 6.2; 256^2 cavity 26.7 -> 8.2;
+  // 512x1024 D2Q16 22.6 -> 16.4; 512^2 D2Q36 139 -> 20.5, D3Q64 34.9 -> 18.5).
+  // From two waves of `large` rows on, `large` is taken: 16 to 128 rows are
+  // within 3% there (4096^2 D2Q16: 368, 357, 364, 367 us at 16, 32, 64, 128;
+  // D3Q64: 808, 775, 777, 770).
+  constexpr double kPro = 1.5;
+  const bool comp = h->p.storage == LESBGK_F32C, wide = h->q >= 32;
+  const double slots = wide ? 2 : comp ? 3 : 4;  // blocks an SM holds (registers)
+  const double share = wide ? 0.85 : comp ? 0.70 : 0.63;
+  const int large = wide && !comp ? 128 : 32;
   h->cpt = 1;
   const int nstrips = (nx + 27) / 28;
-  const int rows_default = h->q >= 36 ? 128 : 32;
-  if (h->rows <= 0) h->rows = ny < rows_default ? ny : rows_default;
+  if (h->rows <= 0) {
+    const double sms = h->sm_count > 0 ? h->sm_count : 152;
+    const double cap = slots * sms, full = share * slots;
+    const double per_block = h->q >= 100 ? 1 : kBlock / 32;  // strips (D3Q216: one)
+    h->rows = large < ny ? large : ny;
+    if ((double)nstrips * ny < 2.0 * large * cap * per_block) {
+      double best = 0.0;
+      for (int r = 1; r <= (wide ? 128 : 64) && r <= ny; ++r) {
+        const int rest = ny % r;  // rows of a last, shorter segment
+        const double whole = std::ceil(nstrips * (double)(ny / r) / per_block);
+        const double blocks = std::ceil(nstrips * (double)((ny + r - 1) / r) / per_block);
+        double t;
+        if (blocks <= cap) t = (r + kPro) * std::fmax(1.0, share * std::ceil(blocks / sms));
+        else if (whole <= cap) t = (r + kPro) * full + rest + kPro;  // the short segments follow the full wave
+        else t = full * (r + kPro) * (blocks / cap + 0.5);
+        if (r == 1 || t <= best) {
+          best = t;
+          h->rows = r;
+        }
+      }
+    }
+  }
   h->args.rows = h->rows;
   h->args.nstrips = nstrips;
   h->args.nseg = (ny + h->rows - 1) / h->rows;

@@ -1,0 +1,41 @@
+"""The default launch shape (rows per segment from the grid's size): the same
+bits as fixed segments, at sizes on both sides of the rule's lines."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1209_6548_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+# sizes: one row, rows short of a segment, an even wave, past one wave, and
+# past two waves of the longest segments (the fixed shape)
+SIZES = [(4, 2), (4, 65), (29, 3), (257, 255), (530, 513), (1030, 1021), (2053, 2049)]
+
+
+@pytest.mark.parametrize("nx,ny", SIZES)
+@pytest.mark.parametrize("nroots,dim,storage", [(4, 2, 0), (4, 2, 2), (4, 2, 3), (6, 2, 0), (4, 3, 0), (6, 3, 0)])
+def test_default_rows_give_the_bits_of_fixed_rows(nx, ny, nroots, dim, storage):
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    if nx * ny * nroots ** dim > 2 ** 26 and (nroots, dim, storage) != (4, 2, 0):
+        pytest.skip("large grids with the base set only")
+    prob = I.Problem(name="shape", nroots=nroots, dim=dim, nx=nx, ny=ny, bc_y=I.DIFFUSE, kn=0.1, b=-0.5,
+                     scheme=I.SPLIT, wall_ux=(0.0, 0.05), g=(1e-3, 0.0))
+    p = L.params_from_problem(prob)
+    p.storage = storage
+    init = I.random_fields(prob, seed=nx + ny)
+    got = []
+    for rows in (0, 7, ny):
+        s = L.Solver(p, h_init=init)
+        if rows:
+            s.set_launch(0, rows)
+        s.step(3)
+        got.append((s.populations(), s.info.rows_per_segment))
+    assert 1 <= got[0][1] <= ny and got[1][1] == 7 and got[2][1] == ny
+    assert np.isfinite(float(got[0][0].double().sum()))
+    for other, _ in got[1:]:
+        assert torch.equal(got[0][0], other)
