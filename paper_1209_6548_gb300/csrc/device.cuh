@@ -162,6 +162,12 @@ __device__ __forceinline__ float xflux(bool right, float x, float kx, const NB &
   return fmaf(-kx, nb.right(sg) - sg, dr);
 }
 
+// Programmatic dependent launch: a step's blocks may start while the previous
+// step's last ones run; pdl_wait returns when that kernel has finished and its
+// stores are visible, pdl_trigger lets the next step's blocks in.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // neighbour lanes of a warp-wide strip
 struct StripLanes {
   __device__ __forceinline__ float left(float v) const { return __shfl_up_sync(kFull, v, 1); }
@@ -818,6 +824,15 @@ template <int NR, class S, int Q, class TT>
 __device__ __forceinline__ void ld_group_s(const S *p, long long gstride, int g, float (&F)[Q], const TT &Tt) {
   using R = typename Raw<LayoutQ<NR, S, Q>::VB>::T;
   const R raw = __ldg(reinterpret_cast<const R *>(p + g * gstride));
+  unpack_group<NR, S>(raw, g, F, Tt);
+}
+
+// The same past L1 (and never through the read-only path): for buffers that
+// the previous kernel may still have been writing when this one started.
+template <int NR, class S, int Q, class TT>
+__device__ __forceinline__ void ld_group_cg(const S *p, long long gstride, int g, float (&F)[Q], const TT &Tt) {
+  using R = typename Raw<LayoutQ<NR, S, Q>::VB>::T;
+  const R raw = __ldcg(reinterpret_cast<const R *>(p + g * gstride));
   unpack_group<NR, S>(raw, g, F, Tt);
 }
 

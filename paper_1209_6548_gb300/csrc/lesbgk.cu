@@ -81,16 +81,18 @@ __global__ void __launch_bounds__(kBlock) k_step(const S *__restrict__ fin, S *_
   // y-stencil state per population:
   //   c_y > 0: s0 = f_j - f_{j-1}, s1 = sigma_{j-1}; fc = f_j
   //   c_y < 0: s0 = f_{j+1},       s1 = sigma_j;     fc = f_j
+  pdl_wait();
+  pdl_trigger();
   float fc[Q], s0[Q], s1[Q];
   {
     float m2[Q], m1[Q], p1[Q];
     const S *pm2 = row_ptr(y0 - 2), *pm1 = row_ptr(y0 - 1), *pz = row_ptr(y0), *pp1 = row_ptr(y0 + 1);
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      ld_group_s<NR, S>(pm1, gstride, g, m1, A);
-      ld_group_s<NR, S>(pz, gstride, g, fc, A);
-      if (g >= G / 2) ld_group_s<NR, S>(pm2, gstride, g, m2, A);
-      else ld_group_s<NR, S>(pp1, gstride, g, p1, A);
+      ld_group_cg<NR, S>(pm1, gstride, g, m1, A);
+      ld_group_cg<NR, S>(pz, gstride, g, fc, A);
+      if (g >= G / 2) ld_group_cg<NR, S>(pm2, gstride, g, m2, A);
+      else ld_group_cg<NR, S>(pp1, gstride, g, p1, A);
     }
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
@@ -288,10 +290,12 @@ __global__ void __launch_bounds__(kBlockZ) k_step_z(const S *__restrict__ fin, S
     }
   };
   auto load_z = [&](const S *p, int g, float (&F)[Q]) {
-    const T raw = __ldg(reinterpret_cast<const T *>(p + g * gstride));
+    const T raw = __ldcg(reinterpret_cast<const T *>(p + g * gstride));
     unpack_z(raw, g, F);
   };
 
+  pdl_wait();
+  pdl_trigger();
   float fc[Q], s0[Q], s1[Q];
   {
     float m2[Q], m1[Q], p1[Q];
@@ -614,13 +618,15 @@ __global__ void __launch_bounds__(kBlock, NZ == 1 ? 3 : 1) k_step_c(const float 
     const uint4 *p = vx + (long long)map_row(j, ny, A.walls) * nx;
     uint4 v[G];
 #pragma unroll
-    for (int g = 0; g < G; ++g) v[g] = __ldg(p + g * plane);
+    for (int g = 0; g < G; ++g) v[g] = __ldcg(p + g * plane);
     unpack(v, hi, lo);
   };
 
   // y-stencil per population, as in k_step, with hi and lo parts of values:
   //   c_y > 0: s0 = f_j - f_{j-1} (a difference), s1 = sigma_{j-1}; fc = f_j
   //   c_y < 0: s0 = f_{j+1} (s0h + s0l),        s1 = sigma_j;     fc = f_j
+  pdl_wait();
+  pdl_trigger();
   float fch[Q], fcl[Q], s0h[Q], s0l[Q], s1[Q];
   {
     float m2h[Q], m2l[Q], m1h[Q], m1l[Q], p1h[Q], p1l[Q];
@@ -1102,10 +1108,10 @@ int pick_launch(lesbgk *h) {
   // of that latency); past one wave the blocks' ends are spread over half a
   // segment.  Small grids so get short segments, middle ones the longest that
   // fill every SM evenly (us per step with 32 or, D2Q36 and D3Q216, 128 rows ->
-  // now; 4x64 D2Q16 20.5 -> 4.1, D2Q36 69.7 -> 6.2; 256^2 cavity 26.7 -> 8.2;
-  // 512x1024 D2Q16 22.6 -> 16.4; 512^2 D2Q36 139 -> 20.5, D3Q64 34.9 -> 18.5).
+  // now; 4x64 D2Q16 18.6 -> 2.7, D2Q36 70 -> 4.2; 256^2 cavity 25.6 -> 4.9;
+  // 512x1024 D2Q16 19.8 -> 14.8; 512^2 D2Q36 140 -> 18.0, D3Q64 33.0 -> 15.5).
   // From two waves of `large` rows on, `large` is taken: 16 to 128 rows are
-  // within 3% there (4096^2 D2Q16: 368, 357, 364, 367 us at 16, 32, 64, 128;
+  // within 4% there (4096^2 D2Q16: 367, 354, 361, 365 us at 16, 32, 64, 128;
   // D3Q64: 808, 775, 777, 770).
   constexpr double kPro = 1.5;
   const bool comp = h->p.storage == LESBGK_F32C, wide = h->q >= 32;
@@ -1125,8 +1131,13 @@ int pick_launch(lesbgk *h) {
         const int rest = ny % r;  // rows of a last, shorter segment
         const double whole = std::ceil(nstrips * (double)(ny / r) / per_block);
         const double blocks = std::ceil(nstrips * (double)((ny + r - 1) / r) / per_block);
-        double t;
-        if (blocks <= cap) t = (r + kPro) * std::fmax(1.0, share * std::ceil(blocks / sms));
+        double t, k = std::ceil(blocks / sms);
+        // the next step's blocks enter as slots free up (launch_step): with more
+        // than half of an SM's slots taken they do not spread evenly, and some
+        // SM gets a full set (1024^2 compensated: two of three slots, 32 rows,
+        // 56 us per step; three of three, 21 rows, 40 us)
+        if (2.0 * k > slots) k = slots;
+        if (blocks <= cap) t = (r + kPro) * std::fmax(1.0, share * k);
         else if (whole <= cap) t = (r + kPro) * full + rest + kPro;  // the short segments follow the full wave
         else t = full * (r + kPro) * (blocks / cap + 0.5);
         if (r == 1 || t <= best) {
@@ -1249,45 +1260,63 @@ int launch_step(lesbgk *h, const void *fin, void *fout, cudaStream_t s) {
     using E = typename Elem<S>::T;
     const E *fi = static_cast<const E *>(fin);
     E *fo = static_cast<E *>(fout);
+    // Each step may be scheduled while the previous one still runs (the kernels
+    // wait for it before their first load): hides the launch and the drain,
+    // about 2.5 us of every step (us per step, before -> now: 4x64 4.1 -> 2.7,
+    // 256^2 cavity 8.2 -> 5.0, 512x1024 16.4 -> 14.8, 1024^2 31.8 -> 29.1,
+    // 4096^2 356.8 -> 354.3)
+    auto go = [&](auto kernel, unsigned blocks, unsigned threads, size_t smem) {
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at.val.programmaticStreamSerializationAllowed = 1;
+      cudaLaunchConfig_t c{};
+      c.gridDim = dim3(blocks);
+      c.blockDim = dim3(threads);
+      c.dynamicSmemBytes = smem;
+      c.stream = s;
+      c.attrs = &at;
+      c.numAttrs = 1;
+      cudaLaunchKernelEx(&c, kernel, fi, fo, h->args);
+    };
     const bool split = h->p.scheme == LESBGK_SPLIT;
     if constexpr (kIsComp<S>) {  // compensated storage: hi + lo planes
       constexpr size_t smem = step_smem_bytes<NR, S, NZ>();
-      if (split) k_step_c<true, kRing, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
-      else k_step_c<false, kRing, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
+      if (split) go(k_step_c<true, kRing, NZ>, grid, kBlock, smem);
+      else go(k_step_c<false, kRing, NZ>, grid, kBlock, smem);
       return;
     } else if constexpr (NZ == 3) {  // D3Q216: a block of three warps per strip and segment
       constexpr size_t smem = stepz_smem_bytes<kRing, S>();
       const unsigned gz = (unsigned)warps;
       const int wm = h->args.xwalls ? 2 : (h->args.walls && h->args.wspec != 0.0f ? 1 : 0);
       if (wm == 2) {  // walls in x
-        if (split) k_step_z<true, kRing, 2, S><<<gz, kBlockZ, smem, s>>>(fi, fo, h->args);
-        else k_step_z<false, kRing, 2, S><<<gz, kBlockZ, smem, s>>>(fi, fo, h->args);
+        if (split) go(k_step_z<true, kRing, 2, S>, gz, kBlockZ, smem);
+        else go(k_step_z<false, kRing, 2, S>, gz, kBlockZ, smem);
         return;
       }
       if (split) {
-        if (wm == 1) k_step_z<true, kRing, 1, S><<<gz, kBlockZ, smem, s>>>(fi, fo, h->args);
-        else k_step_z<true, kRing, 0, S><<<gz, kBlockZ, smem, s>>>(fi, fo, h->args);
+        if (wm == 1) go(k_step_z<true, kRing, 1, S>, gz, kBlockZ, smem);
+        else go(k_step_z<true, kRing, 0, S>, gz, kBlockZ, smem);
       } else {
-        if (wm == 1) k_step_z<false, kRing, 1, S><<<gz, kBlockZ, smem, s>>>(fi, fo, h->args);
-        else k_step_z<false, kRing, 0, S><<<gz, kBlockZ, smem, s>>>(fi, fo, h->args);
+        if (wm == 1) go(k_step_z<false, kRing, 1, S>, gz, kBlockZ, smem);
+        else go(k_step_z<false, kRing, 0, S>, gz, kBlockZ, smem);
       }
       return;
     } else {
       constexpr size_t smem = step_smem_bytes<NR, S, NZ>();
       if (h->args.xwalls) {  // walls in x (cavity)
-        if (split) k_step<NR, N, true, kRing, S, 2, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
-        else k_step<NR, N, false, kRing, S, 2, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
+        if (split) go(k_step<NR, N, true, kRing, S, 2, NZ>, grid, kBlock, smem);
+        else go(k_step<NR, N, false, kRing, S, 2, NZ>, grid, kBlock, smem);
         return;
       }
       if constexpr (std::is_same<S, float>::value) {  // Maxwell walls: FP32 storage (checked at set-up)
         if (h->args.walls && h->args.wspec != 0.0f) {  // Maxwell walls
-          if (split) k_step<NR, N, true, kRing, S, 1, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
-          else k_step<NR, N, false, kRing, S, 1, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
+          if (split) go(k_step<NR, N, true, kRing, S, 1, NZ>, grid, kBlock, smem);
+          else go(k_step<NR, N, false, kRing, S, 1, NZ>, grid, kBlock, smem);
           return;
         }
       }
-      if (split) k_step<NR, N, true, kRing, S, 0, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
-      else k_step<NR, N, false, kRing, S, 0, NZ><<<grid, kBlock, smem, s>>>(fi, fo, h->args);
+      if (split) go(k_step<NR, N, true, kRing, S, 0, NZ>, grid, kBlock, smem);
+      else go(k_step<NR, N, false, kRing, S, 0, NZ>, grid, kBlock, smem);
     }
   });
   return 0;
