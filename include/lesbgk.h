@@ -350,16 +350,19 @@ int lesbgk_batch_get_info(const lesbgk_batch *b, int32_t slot, lesbgk_info *out)
 int lesbgk_batch_raw_bytes(const lesbgk_batch *b, int32_t slot, size_t *bytes);
 int lesbgk_batch_get_raw(lesbgk_batch *b, int32_t slot, void *d_out, void *stream);
 int lesbgk_batch_set_raw(lesbgk_batch *b, int32_t slot, const void *d_in, int64_t steps_done, void *stream);
-/* Rows per work item (default 32); results do not depend on it. */
+/* Rows per work item; until it is set (or lesbgk_batch_autotune called) the
+ * rows follow the solves in the batch.  Results do not depend on it. */
 int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream);
-/* Resident kernel (on by default): D2Q16 FP32 instances of at most max_ny rows
+/* Resident kernel: D2Q16 FP32 instances of at most max_ny rows
  * (0 keeps the current limit, 128 by default) whose two population buffers
  * fit in one block's shared memory (454 rows at nx = 4 on GB300) are each held
  * (steady walls) by one block for steps_per_launch time steps (an even divisor of 64; 0
  * keeps the current, 64 by default), reading and writing device memory once
  * per launch, while the other instances take one launch per step; in the
  * 64-step graphs the two run side by side.  A resident instance is one
- * block's serial work, so tall ones are better left to the per-step kernel.
+ * block's serial work, so tall ones are better left to the per-step kernel:
+ * until this call (or lesbgk_batch_autotune) it is on where every solve of
+ * the batch has at most 64 rows, and off otherwise.
  * Results do not depend on the choice (bitwise). */
 int lesbgk_batch_set_resident(lesbgk_batch *b, int32_t on, int32_t steps_per_launch, int32_t max_ny, void *stream);
 /* The launch configuration in use (any pointer may be NULL). */

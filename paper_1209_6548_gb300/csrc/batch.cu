@@ -40,8 +40,15 @@ constexpr int kBRing = 4;
 // kernels carry the FP64 wall-table code, the others none of it)
 constexpr int kNumClasses = 18;
 constexpr int kGraphSteps = 64;
+constexpr int kChains = 4;  // at most: independent chains of steps a class's solves are dealt to
 constexpr size_t kGuardBytes = 256;       // guard words after each slot's pool block
 constexpr unsigned char kGuardByte = 0xA5;
+// a batch whose solves all have at most this many rows goes to the resident
+// kernel by default (64 channels, us per step, per-step kernel against
+// resident: up to 32 rows 2.8 and 1.1, up to 64 rows 2.9 and 2.1, up to 128
+// rows 3.1 and 3.7); beside taller ones, whose steps set the pace, it only
+// takes their slots (256 channels up to 512 rows: 6.5 and 6.7)
+constexpr int kAutoResidentNy = 64;
 constexpr int kBuckets = 6;  // resident instances by height: ny <= 16, 32, ..., 512 (smem permitting)
 
 // Per-instance descriptor (device memory).
@@ -81,10 +88,18 @@ struct InstRegs {
   int vmode, has_force;
 };
 
+// The coefficients of a lane group in shared memory, 16-byte entries: the
+// advection's pair operands, NR of {kx, kx, -ax, -ax} (ix), NR/2 of
+// {ky, ky', -ay, -ay'} (the pair iy, iy + 1, iy even) and NR/2 of {-ay, -ay'}
+// for the x-sweep's input (0 in the printed update, whose x-fluxes take f^n
+// itself), then the scalars of InstRegs in two, {ny, walls, 0, instance} and
+// {output pointer, rows, first row}.
+template <int NR>
+constexpr int kCoefs = 2 * NR + 4;
+
 template <int NR, class S = float, int NZ = 1>
-constexpr size_t batch_smem_bytes() {
-  return (size_t)(kBBlock / 32) * kBRing * Layout<NR, S, NZ>::G * 32 * Layout<NR, S, NZ>::VB;
-}
+constexpr size_t kBatchRingBytes =
+    (size_t)(kBBlock / 32) * kBRing * Layout<NR, S, NZ>::G * 32 * Layout<NR, S, NZ>::VB;
 
 // neighbour lanes inside a lane group of W lanes (periodic in x)
 struct GroupLanes {
@@ -126,8 +141,14 @@ __device__ __forceinline__ void wall_fix_heated(float (&O)[Q], int side, const T
 // One time step of every work item of a class (velocity set and storage S:
 // FP32 deviations, or FP16/BF16 relative deviations rounded stochastically
 // with the random words of k_step, keyed by the instance's step count and row).
+// What bounds it: issue (D2Q16: 740 instructions per node and step in short items,
+// 600 in long ones: 553k nodes cannot take less than 8.5 us on 152 SMs) and the latency of each warp's
+// chain, so it needs warps: the per-item coefficients and flags sit in shared
+// memory (a dozen 16-byte reads per row) instead of registers, which lets
+// D2Q16 keep four blocks on an SM (165 -> 128 registers) and D2Q36 run
+// without spills (96 B before), on packed pairs.
 template <int NR, int N, int W, class S, bool HEAT, int NZ>
-__global__ void __launch_bounds__(kBBlock) k_batch_step(const BatchArgs B, const int par) {
+__global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_step(const BatchArgs B, const int par) {
   using Lay = Layout<NR, S, NZ>;
   constexpr int Q = Lay::Q, H = Lay::H, V = Lay::V, G = Lay::G;
   constexpr int GPW = 32 / W;
@@ -143,40 +164,58 @@ __global__ void __launch_bounds__(kBBlock) k_batch_step(const BatchArgs B, const
   const WorkItem wi = B.items[first + it];
   const InstDesc &D = B.desc[wi.inst];
   const int ny = D.ny, walls = D.walls;
-  const bool split = D.split != 0;
-  InstRegs P{D.c_omega, D.visc_pow, D.b, D.beta, D.dtgx, D.dtgy, D.vmode, D.has_force};
-  float ax[NR], kx[NR], ay[NR], ky[NR];
-#pragma unroll
-  for (int i = 0; i < NR; ++i) {
-    ax[i] = D.ax[i];
-    kx[i] = D.kx[i];
-    ay[i] = D.ay[i];
-    ky[i] = D.ky[i];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  // this group's coefficients: entry c at coef[c * GPW], one broadcast per group
+  float4 *coef = reinterpret_cast<float4 *>(smem_raw + kBatchRingBytes<NR, S, NZ>) +
+                 (threadIdx.x >> 5) * kCoefs<NR> * GPW + gi;
+  for (int c = lx; c < kCoefs<NR>; c += W) {
+    float4 v;
+    if (c < NR) {
+      v = make_float4(D.kx[c], D.kx[c], -D.ax[c], -D.ax[c]);
+    } else if (c < NR + NR / 2) {
+      const int iy = 2 * (c - NR);
+      v = make_float4(D.ky[iy], D.ky[iy + 1], -D.ay[iy], -D.ay[iy + 1]);
+    } else if (c < 2 * NR) {
+      const int iy = 2 * (c - NR - NR / 2);
+      v = D.split ? make_float4(-D.ay[iy], -D.ay[iy + 1], 0.f, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if (c == 2 * NR) {
+      v = make_float4(D.c_omega, D.visc_pow, D.b, D.beta);
+    } else if (c == 2 * NR + 1) {
+      v = make_float4(D.dtgx, D.dtgy, __int_as_float(D.vmode), __int_as_float(D.has_force));
+    } else if (c == 2 * NR + 2) {
+      v = make_float4(__int_as_float(ny), __int_as_float(walls), 0.f, __int_as_float(wi.inst));
+    } else {
+      const unsigned long long o = reinterpret_cast<unsigned long long>(D.f[par ^ 1]);
+      v = make_float4(__int_as_float((int)(unsigned)o), __int_as_float((int)(unsigned)(o >> 32)),
+                      __int_as_float(live ? wi.rows : 0), __int_as_float(wi.y0));
+    }
+    coef[c * GPW] = v;
   }
+  __syncwarp();
   const S *fin = reinterpret_cast<const S *>(D.f[par]);
-  S *fout = reinterpret_cast<S *>(D.f[par ^ 1]);
   const long long gstride = (long long)V * W * ny;
   const long long rstride = (long long)V * W;
   const S *fx = fin + (long long)lx * V;
   const int y0 = wi.y0;
-  const int rows = live ? wi.rows : 0;
-  int nrows = rows;  // the warp runs its longest item's rows
+  int nrows = live ? wi.rows : 0;  // the warp runs its longest item's rows
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) nrows = max(nrows, __shfl_xor_sync(kFull, nrows, o));
   const int srcL = gi * W + ((lx + W - 1) & (W - 1));
   const int srcR = gi * W + ((lx + 1) & (W - 1));
   auto row_ptr = [&](int j) { return fx + map_row(j, ny, walls) * rstride; };
 
+  pdl_wait();  // the tables above are the host's; the populations are the previous step's
+  pdl_trigger();
   float fc[Q], s0[Q], s1[Q];
   {
     float m2[Q], m1[Q], p1[Q];
     const S *pm2 = row_ptr(y0 - 2), *pm1 = row_ptr(y0 - 1), *pz = row_ptr(y0), *pp1 = row_ptr(y0 + 1);
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      ld_group_s<NR, S>(pm1, gstride, g, m1, B.lat);
-      ld_group_s<NR, S>(pz, gstride, g, fc, B.lat);
-      if (g >= G / 2) ld_group_s<NR, S>(pm2, gstride, g, m2, B.lat);
-      else ld_group_s<NR, S>(pp1, gstride, g, p1, B.lat);
+      ld_group_cg<NR, S>(pm1, gstride, g, m1, B.lat);
+      ld_group_cg<NR, S>(pz, gstride, g, fc, B.lat);
+      if (g >= G / 2) ld_group_cg<NR, S>(pm2, gstride, g, m2, B.lat);
+      else ld_group_cg<NR, S>(pp1, gstride, g, p1, B.lat);
     }
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
@@ -190,18 +229,21 @@ __global__ void __launch_bounds__(kBBlock) k_batch_step(const BatchArgs B, const
     }
   }
 
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   using T = typename Raw<Lay::VB>::T;
   T *ring = reinterpret_cast<T *>(smem_raw) + (size_t)(threadIdx.x >> 5) * kBRing * G * 32 + lane;
   int r1 = map_row(y0 + 1, ny, walls), r2 = map_row(y0 + 2, ny, walls);
+  const int4 *iflags = reinterpret_cast<const int4 *>(coef + (2 * NR + 2) * GPW);
+  const int4 *iout = reinterpret_cast<const int4 *>(coef + (2 * NR + 3) * GPW);
   auto issue_rowload = [&](int k) {
     if (k < nrows) {
+      const int2 fl = *reinterpret_cast<const int2 *>(iflags);  // ny, walls
+      const long long gstride = (long long)(V * W) * fl.x;
       const S *q1 = fx + r1 * rstride, *q2 = fx + r2 * rstride;
       T *slot = ring + (k % kBRing) * G * 32;
 #pragma unroll
       for (int g = 0; g < G; ++g) cp_async_raw<Lay::VB>(slot + g * 32, (g >= G / 2 ? q1 : q2) + g * gstride);
       r1 = r2;
-      r2 = r2 + 1 < ny ? r2 + 1 : (walls ? ny - 1 : 0);
+      r2 = r2 + 1 < fl.x ? r2 + 1 : (fl.y ? fl.x - 1 : 0);
     }
     cp_async_commit();
   };
@@ -209,7 +251,6 @@ __global__ void __launch_bounds__(kBBlock) k_batch_step(const BatchArgs B, const
   for (int k = 0; k < kBRing - 1; ++k) issue_rowload(k);
 
   for (int k = 0; k < nrows; ++k) {
-    const int j = y0 + k;
     issue_rowload(k + kBRing - 1);
     cp_async_wait<kBRing - 1>();
     float ld[Q];
@@ -220,53 +261,62 @@ __global__ void __launch_bounds__(kBBlock) k_batch_step(const BatchArgs B, const
     }
     float acc[Q];
     float omw;
-    collide_any<NR, N>(fc, acc, omw, B.lat, P);
+    {
+      const float4 p = coef[2 * NR * GPW], q = coef[(2 * NR + 1) * GPW];
+      const InstRegs P{p.x, p.y, p.z, p.w, q.x, q.y, __float_as_int(q.z), __float_as_int(q.w)};
+      collide_any<NR, N>(fc, acc, omw, B.lat, P);
+    }
     float xs[Q];
     const GroupLanes nb{srcL, srcR};
-    if constexpr (NR == 4) {  // packed pairs a, a+1 (same ix, c_y of one sign)
-      const float2 omw2 = make_float2(omw, omw);
+    const float2 omw2 = make_float2(omw, omw);
+    const int4 fl = *iflags;
 #pragma unroll
-      for (int a = 0; a < Q; a += 2) {
-        const int iy = a % NR;
-        const float2 nay = make_float2(-ay[iy], -ay[iy + 1]);
-        float2 f0;
-        const float2 diff = yflux2(iy >= H, a, fc, s0, s1, ld, make_float2(ky[iy], ky[iy + 1]), f0);
-        const float2 ac = fma2(omw2, f0, fma2(nay, diff, make_float2(acc[a], acc[a + 1])));
-        const float2 x2 = split ? fma2(nay, diff, f0) : f0;
-        acc[a] = ac.x;
-        acc[a + 1] = ac.y;
-        xs[a] = x2.x;
-        xs[a + 1] = x2.y;
-      }
+    for (int a = 0; a < Q; a += 2) {  // packed pairs a, a+1 (same ix)
+      const int iy = a % NR;
+      const float4 cy = coef[(NR + iy / 2) * GPW];
+      const float2 nays = *reinterpret_cast<const float2 *>(coef + (NR + NR / 2 + iy / 2) * GPW);
+      const float2 ky = make_float2(cy.x, cy.y), nay = make_float2(cy.z, cy.w);
+      if ((iy >= H) != (iy + 1 >= H)) {  // a pair across c_y = 0 (D2Q36): one at a time
 #pragma unroll
-      for (int a = 0; a < Q; a += 2) {
-        const int ix = (a / NR) % NR;
-        const float2 nax = make_float2(-ax[ix], -ax[ix]);
-        const float2 diff = xflux2(ix >= H, make_float2(xs[a], xs[a + 1]), make_float2(kx[ix], kx[ix]), nb);
-        const float2 ac = fma2(nax, diff, make_float2(acc[a], acc[a + 1]));
-        acc[a] = ac.x;
-        acc[a + 1] = ac.y;
+        for (int b = a; b < a + 2; ++b) {
+          float f0;
+          const float diff = yflux(b % NR >= H, b, fc, s0, s1, ld, b == a ? ky.x : ky.y, f0);
+          acc[b] = fmaf(omw, f0, fmaf(b == a ? nay.x : nay.y, diff, acc[b]));
+          xs[b] = fmaf(b == a ? nays.x : nays.y, diff, f0);
+        }
+        continue;
       }
-    } else {  // D2Q36: one population at a time (the pair constants would spill)
-#pragma unroll
-      for (int a = 0; a < Q; ++a) {
-        const int iy = a % NR;
-        float f0;
-        const float diff = yflux(iy >= H, a, fc, s0, s1, ld, ky[iy], f0);
-        acc[a] = fmaf(omw, f0, fmaf(-ay[iy], diff, acc[a]));
-        xs[a] = split ? fmaf(-ay[iy], diff, f0) : f0;
-      }
-#pragma unroll
-      for (int a = 0; a < Q; ++a) {
-        const int ix = (a / NR) % NR;
-        acc[a] = fmaf(-ax[ix], xflux(ix >= H, xs[a], kx[ix], nb), acc[a]);
-      }
+      float2 f0;
+      const float2 diff = yflux2(iy >= H, a, fc, s0, s1, ld, ky, f0);
+      const float2 ac = fma2(omw2, f0, fma2(nay, diff, make_float2(acc[a], acc[a + 1])));
+      const float2 x2 = fma2(nays, diff, f0);
+      acc[a] = ac.x;
+      acc[a + 1] = ac.y;
+      xs[a] = x2.x;
+      xs[a + 1] = x2.y;
     }
-    if (walls && (j == 0 || j == ny - 1)) {
+#pragma unroll
+    for (int ix = 0; ix < NR; ++ix) {
+      const float4 cx = coef[ix * GPW];
+      const float2 kx = make_float2(cx.x, cx.y), nax = make_float2(cx.z, cx.w);
+#pragma unroll
+      for (int a0 = ix * NR; a0 < Q; a0 += NR * NR)
+#pragma unroll
+        for (int a = a0; a < a0 + NR; a += 2) {
+          const float2 diff = xflux2(ix >= H, make_float2(xs[a], xs[a + 1]), kx, nb);
+          const float2 ac = fma2(nax, diff, make_float2(acc[a], acc[a + 1]));
+          acc[a] = ac.x;
+          acc[a + 1] = ac.y;
+        }
+    }
+    const int4 out = *iout;
+    const int j = out.w + k;
+    if (fl.y && (j == 0 || j == fl.x - 1)) {
       const int side = j == 0 ? 0 : 1;
+      const InstDesc &D = B.desc[fl.w];
       if constexpr (HEAT) {  // the wall temperature of the time this step writes
         const HeatPoly &hp = *D.heat;
-        const double hv = wall_heating(hp, (double)(B.nstep[2 * wi.inst + par] + 1) * hp.dt);
+        const double hv = wall_heating(hp, (double)(B.nstep[2 * fl.w + par] + 1) * hp.dt);
         if (D.wspec != 0.0f) wall_fix_heated<NR, true>(acc, side, B.lat, hp, hv, D.wspec);
         else wall_fix_heated<NR, false>(acc, side, B.lat, hp, hv, D.wspec);
       } else if (D.wspec != 0.0f) {
@@ -275,10 +325,12 @@ __global__ void __launch_bounds__(kBBlock) k_batch_step(const BatchArgs B, const
         wall_fix<NR, false>(acc, side, B.lat, D);
       }
     }
-    if (k < rows) {
+    if (k < out.z) {
+      const long long gstride = (long long)(V * W) * fl.x;
+      S *fout = reinterpret_cast<S *>((unsigned long long)(unsigned)out.x | (unsigned long long)(unsigned)out.y << 32);
       S *o = fout + (long long)j * rstride + (long long)lx * V;
       if constexpr (Store<S>::kScaled) {  // the key of k_step: step count and row
-        const unsigned seed = (unsigned)B.nstep[2 * wi.inst + par] * 0x9e3779b9u + 0x7f4a7c15u;
+        const unsigned seed = (unsigned)B.nstep[2 * fl.w + par] * 0x9e3779b9u + 0x7f4a7c15u;
         const unsigned key = mix32(seed ^ mix32((unsigned)j));
 #pragma unroll
         for (int g = 0; g < G; ++g) st_group_sr<NR, S>(o, gstride, g, acc, B.lat, key);
@@ -293,7 +345,7 @@ __global__ void __launch_bounds__(kBBlock) k_batch_step(const BatchArgs B, const
   // rounding) follows its state into the other buffer: one thread per
   // instance, while every thread of this launch reads parity par only
   if constexpr (HEAT || Store<S>::kScaled)
-    if (live && wi.y0 == 0 && lx == 0) B.nstep[2 * wi.inst + (par ^ 1)] = B.nstep[2 * wi.inst + par] + 1;
+    if (iout->z && iout->w == 0 && lx == 0) B.nstep[2 * iflags->w + (par ^ 1)] = B.nstep[2 * iflags->w + par] + 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -681,7 +733,7 @@ struct lesbgk_batch {
   int capacity = 0, nx = 0, W = 0;
   InstDesc *d_desc = nullptr;
   WorkItem *d_items = nullptr;
-  int *d_range = nullptr;      // {first, count} per class of the items the per-step kernel takes
+  int *d_range = nullptr;      // {first, count} per class of the items the per-step kernel takes, then per class and chain
   int *d_range_all = nullptr;  // {first, count} per class of all items (residuals, moments)
   int *d_rlist = nullptr;      // resident instances, bucket after bucket
   int *d_rrange = nullptr;     // {first, count} per bucket
@@ -703,15 +755,19 @@ struct lesbgk_batch {
   bool resident = true;      // D2Q16 instances that fit in shared memory take the resident kernel
   int resident_k = 64;       // time steps per resident launch (divides kGraphSteps)
   int resident_ny = 0;       // tallest instance the resident kernel can hold (shared memory)
-  int resident_limit = 128;  // tallest instance it takes (autotuned: a tall one is one block's serial work)
+  int resident_limit = 128;  // tallest instance it takes (a tall one is one block's serial work)
+  bool auto_resident = true;  // until the caller chooses: only where every solve is that short
   int graph_rgrid[kBuckets] = {};
-  int rows = 32;
+  int rows = 32;           // rows per work item where the caller sets them
+  bool auto_rows = true;   // until then: rows and chains per class by pick_rows
+  int rows_of[kNumClasses] = {}, chains_of[kNumClasses] = {};
   int par = 0;
   int sm_count = 0;
   LatTables lat[kNumClasses];
   bool lat_ready[kNumClasses] = {};
   cudaGraphExec_t graph = nullptr;
-  int graph_grid[kNumClasses] = {};
+  int range_chain[kNumClasses][kChains][2] = {};
+  int graph_grid[kNumClasses][kChains] = {};
   bool graph_dirty = true;
   bool items_dirty = false;  // slots changed since the work list was uploaded
 };
@@ -734,7 +790,7 @@ Layout0 fixed_layout(int capacity) {
   L.mass = o;  // per-item mass partial of the residual pass
   o = align_up(o + sizeof(double) * (size_t)capacity * kItemsPerSlot, 256);
   L.range = o;
-  o = align_up(o + sizeof(int) * 2 * kNumClasses, 256);
+  o = align_up(o + sizeof(int) * 2 * kNumClasses * (1 + kChains), 256);
   L.range_all = o;
   o = align_up(o + sizeof(int) * 2 * kNumClasses, 256);
   L.rlist = o;
@@ -799,10 +855,12 @@ void *step_kernel(int cls, int W) {
   return fn;
 }
 
-size_t step_smem(int cls) {
+size_t step_smem(int cls, int W) {
   size_t b = 0;
   with_class(cls, [&](auto r, auto, auto st, auto, auto z) {
-    b = batch_smem_bytes<decltype(r)::value, decltype(st), decltype(z)::value>();
+    constexpr int NR = decltype(r)::value;
+    b = kBatchRingBytes<NR, decltype(st), decltype(z)::value> +
+        (size_t)(kBBlock / 32) * kCoefs<NR> * (32 / W) * sizeof(float4);
   });
   return b;
 }
@@ -863,6 +921,10 @@ cudaError_t launch_resident(lesbgk_batch *b, int K, int p_in, int p_out, cudaStr
   return e;
 }
 
+const int *chain_range(const lesbgk_batch *b, int cls, int chain) {
+  return b->d_range + 2 * (kNumClasses + cls * kChains + chain);
+}
+
 unsigned step_grid(const lesbgk_batch *b, int n_items) {
   const int gpw = 32 / b->W;
   const long long warps = (n_items + gpw - 1) / gpw;
@@ -870,10 +932,59 @@ unsigned step_grid(const lesbgk_batch *b, int n_items) {
   return (unsigned)std::max<long long>(blocks, 1);
 }
 
-cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, unsigned grid, cudaStream_t s) {
+// One step of a class, or of one of its chains.
+cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s, int chain = -1) {
   BatchArgs a = make_args(b, cls);
+  if (chain >= 0) a.range = chain_range(b, cls, chain);
+  const unsigned grid = step_grid(b, chain < 0 ? b->range[cls][1] : b->range_chain[cls][chain][1]);
   void *args[] = {&a, &par};
-  return cudaLaunchKernel(step_kernel(cls, b->W), dim3(grid), dim3(kBBlock), args, step_smem(cls), s);
+  cudaLaunchAttribute at{};  // may be scheduled while the previous step runs (the kernel waits for it)
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(kBBlock);
+  c.dynamicSmemBytes = step_smem(cls, b->W);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelExC(&c, step_kernel(cls, b->W), args);
+}
+
+// Rows per work item and chains of each class, from the solves it holds, until
+// the caller sets rows: items for one and a half times the blocks its share of
+// the chip holds (by work: the classes run side by side), dealt to kChains
+// chains once they fill it.  A step's launch, first loads and last blocks cost
+// about 4 us whatever its size; beside three other chains that time is filled
+// (512 channels of 16 to 1024 rows, us per step with one chain at its best
+// rows -> four chains at the rule's: D2Q16 17.3 -> 13.8, D2Q36 47.4 -> 42.6,
+// D3Q64 31.9 -> 29.8).  Smaller batches keep one chain (32 channels: 3.3 us
+// against 3.6).  Rows stay while they are within a factor of two of the rule's
+// and the step graph has room, so that admissions seldom rebuild it.
+void pick_rows(lesbgk_batch *b) {
+  double work[kNumClasses] = {}, rows[kNumClasses] = {}, all = 0.0;
+  for (int i = 0; i < b->capacity; ++i) {
+    const auto &sl = b->slots[i];
+    if (!sl.used || is_resident(b, sl)) continue;
+    rows[sl.cls] += sl.p.ny;
+    work[sl.cls] += (double)sl.p.ny * stored_values(sl.p);
+  }
+  for (double w : work) all += w;
+  const double sms = b->sm_count > 0 ? b->sm_count : 152;
+  const double per_block = (double)(kBBlock / b->W);  // items a block takes
+  for (int cls = 0; cls < kNumClasses; ++cls) {
+    if (!(rows[cls] > 0.0)) continue;
+    const double cap = (cls % 3 == 0 ? 4 : 2) * sms * work[cls] / all;
+    int r = b->rows;
+    if (b->auto_rows) r = (int)std::fmin(64.0, std::ceil(rows[cls] / (per_block * 1.5 * cap)));
+    auto chains = [&](int at) { return rows[cls] / (per_block * at) > 0.75 * cap ? kChains : 1; };
+    const int old = b->rows_of[cls];
+    if (b->auto_rows && b->graph && old && 2 * old >= r && old <= 2 * r && b->chains_of[cls] == chains(old) &&
+        rows[cls] / (per_block * old) / b->chains_of[cls] + 1.0 < b->graph_grid[cls][0])
+      continue;
+    b->rows_of[cls] = r;
+    b->chains_of[cls] = chains(r);
+  }
 }
 
 // Rebuild the host work list and copy it with the class ranges to the device:
@@ -882,22 +993,42 @@ cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, unsigned grid, cu
 // residual and moment kernels visit); and the resident instances by bucket.
 int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
   b->items.clear();
+  if (b->auto_resident) {
+    b->resident = true;
+    for (const auto &sl : b->slots)
+      if (sl.used && (sl.cls != 0 || sl.p.ny > std::min(b->resident_ny, kAutoResidentNy))) b->resident = false;
+  }
+  pick_rows(b);
   for (int cls = 0; cls < kNumClasses; ++cls) {
     const int first = (int)b->items.size();
-    std::vector<WorkItem> mine, res;
-    for (int i = 0; i < b->capacity; ++i) {
+    std::vector<WorkItem> mine[kChains], res;
+    // the solves dealt to the chains, the tallest first, each to the shortest
+    std::vector<int> order;
+    for (int i = 0; i < b->capacity; ++i)
+      if (b->slots[i].used && b->slots[i].cls == cls) order.push_back(i);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->slots[x].p.ny > b->slots[y].p.ny; });
+    long long load[kChains] = {};
+    for (int i : order) {
       const auto &sl = b->slots[i];
-      if (!sl.used || sl.cls != cls) continue;
-      auto &dst = is_resident(b, sl) ? res : mine;
-      for (int y0 = 0; y0 < sl.p.ny; y0 += b->rows) dst.push_back({i, y0, std::min(b->rows, sl.p.ny - y0), 0});
+      // (a tall solve keeps within its room of the work list)
+      const int r = std::max(b->rows_of[cls], (int)((sl.p.ny + kItemsPerSlot - 1) / kItemsPerSlot));
+      const int c = (int)(std::min_element(load, load + b->chains_of[cls]) - load);
+      if (!is_resident(b, sl)) load[c] += sl.p.ny;
+      auto &dst = is_resident(b, sl) ? res : mine[c];
+      for (int y0 = 0; y0 < sl.p.ny; y0 += r) dst.push_back({i, y0, std::min(r, sl.p.ny - y0), 0});
     }
-    std::stable_sort(mine.begin(), mine.end(), [](const WorkItem &x, const WorkItem &y) { return x.rows > y.rows; });
-    b->items.insert(b->items.end(), mine.begin(), mine.end());
+    for (int c = 0; c < kChains; ++c) {
+      std::stable_sort(mine[c].begin(), mine[c].end(), [](const WorkItem &x, const WorkItem &y) { return x.rows > y.rows; });
+      b->range_chain[cls][c][0] = (int)b->items.size();
+      b->range_chain[cls][c][1] = (int)mine[c].size();
+      b->items.insert(b->items.end(), mine[c].begin(), mine[c].end());
+    }
+    const int stepped = (int)b->items.size() - first;
     b->items.insert(b->items.end(), res.begin(), res.end());
     b->range[cls][0] = first;
-    b->range[cls][1] = (int)mine.size();
+    b->range[cls][1] = stepped;
     b->range_all[cls][0] = first;
-    b->range_all[cls][1] = (int)(mine.size() + res.size());
+    b->range_all[cls][1] = stepped + (int)res.size();
   }
   if ((long long)b->items.size() > (long long)b->capacity * (long long)kItemsPerSlot)
     return fail(LESBGK_ESPACE, "work list of %zu items exceeds its room", b->items.size());
@@ -915,6 +1046,8 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
   if (!b->items.empty())
     e = cudaMemcpyAsync(b->d_items, b->items.data(), sizeof(WorkItem) * b->items.size(), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_range, b->range, sizeof(b->range), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->d_range + 2 * kNumClasses, b->range_chain, sizeof(b->range_chain), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_range_all, b->range_all, sizeof(b->range_all), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && !rlist.empty())
     e = cudaMemcpyAsync(b->d_rlist, rlist.data(), sizeof(int) * rlist.size(), cudaMemcpyHostToDevice, s);
@@ -924,7 +1057,9 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
   if (e != cudaSuccess) return cuda_fail(e, "work list upload");
   b->items_dirty = false;
   for (int cls = 0; cls < kNumClasses; ++cls)
-    if ((int)step_grid(b, b->range[cls][1]) > b->graph_grid[cls]) b->graph_dirty = true;
+    for (int c = 0; c < kChains; ++c)
+      if (b->range_chain[cls][c][1] && (int)step_grid(b, b->range_chain[cls][c][1]) > b->graph_grid[cls][c])
+        b->graph_dirty = true;
   for (int k = 0; k < kBuckets; ++k)
     if (b->rrange[k][1] > b->graph_rgrid[k]) b->graph_dirty = true;
   return 0;
@@ -938,8 +1073,9 @@ void drop_graph(lesbgk_batch *b) {
   b->graph_dirty = true;
 }
 
-// A graph of kGraphSteps steps: per step one launch per lattice class present,
-// each step after the previous one; grids sized with head room for the
+// A graph of kGraphSteps steps: per class present a chain of one launch per
+// step (the classes step other instances: their chains are independent), each
+// step after the previous one; grids sized with head room for the
 // current work list (kernels read their item counts from device memory, so
 // the graph stays valid while slots come and go).
 int build_graph(lesbgk_batch *b) {
@@ -947,30 +1083,37 @@ int build_graph(lesbgk_batch *b) {
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaGraphCreate(&g, 0);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphCreate");
-  BatchArgs args[kNumClasses];
+  std::vector<BatchArgs> args_store((size_t)kNumClasses * kChains);
+  BatchArgs(*args)[kChains] = reinterpret_cast<BatchArgs(*)[kChains]>(args_store.data());
   int pars[2] = {0, 1};
-  std::vector<cudaGraphNode_t> prev;
+  cudaGraphNode_t prev[kNumClasses][kChains] = {};
+  cudaGraphEdgeData edge{};  // the next step may be scheduled while this one runs
+  edge.from_port = cudaGraphKernelNodePortProgrammatic;
+  edge.type = cudaGraphDependencyTypeProgrammatic;
   for (int cls = 0; cls < kNumClasses; ++cls) {
-    const int n = b->range[cls][1];
-    b->graph_grid[cls] = n ? (int)step_grid(b, n + n / 4 + 64) : 0;
-    args[cls] = make_args(b, cls);
+    for (int c = 0; c < kChains; ++c) {
+      const int n = b->range_chain[cls][c][1];
+      b->graph_grid[cls][c] = n ? (int)step_grid(b, n + n / 4 + 64) : 0;
+      args[cls][c] = make_args(b, cls);
+      args[cls][c].range = chain_range(b, cls, c);
+    }
   }
   for (int st = 0; st < kGraphSteps && e == cudaSuccess; ++st) {
-    std::vector<cudaGraphNode_t> cur;
-    for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls) {
-      if (!b->graph_grid[cls]) continue;
+    for (int k = 0; k < kNumClasses * kChains && e == cudaSuccess; ++k) {
+      const int cls = k / kChains, c = k % kChains;
+      if (!b->graph_grid[cls][c]) continue;
       cudaKernelNodeParams kp{};
-      void *kargs[] = {&args[cls], &pars[st & 1]};
+      void *kargs[] = {&args[cls][c], &pars[st & 1]};
       kp.func = step_kernel(cls, b->W);
-      kp.gridDim = dim3(b->graph_grid[cls]);
+      kp.gridDim = dim3(b->graph_grid[cls][c]);
       kp.blockDim = dim3(kBBlock);
-      kp.sharedMemBytes = (unsigned)step_smem(cls);
+      kp.sharedMemBytes = (unsigned)step_smem(cls, b->W);
       kp.kernelParams = kargs;
       cudaGraphNode_t node;
-      e = cudaGraphAddKernelNode(&node, g, prev.empty() ? nullptr : prev.data(), prev.size(), &kp);
-      cur.push_back(node);
+      e = cudaGraphAddKernelNode(&node, g, nullptr, 0, &kp);
+      if (e == cudaSuccess && st) e = cudaGraphAddDependencies(g, &prev[cls][c], &node, &edge, 1);
+      prev[cls][c] = node;
     }
-    if (!cur.empty()) prev = cur;
   }
   // resident instances: per bucket a chain of kGraphSteps / resident_k launches,
   // each taking resident_k steps in place (an even count: parity 0 to 0),
@@ -1062,7 +1205,7 @@ extern "C" int lesbgk_batch_create(int32_t capacity, int32_t nx, void *d_workspa
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sm_count, cudaDevAttrMultiProcessorCount, dev);
   for (int w : {1, 2, 4, 8, 16, 32})
     for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls)
-      e = cudaFuncSetAttribute(step_kernel(cls, w), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem(cls));
+      e = cudaFuncSetAttribute(step_kernel(cls, w), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem(cls, w));
   // the resident kernel: as tall an instance as two buffers of Q planes fit in
   // the opt-in shared memory of a block
   int optin = 0;
@@ -1071,7 +1214,7 @@ extern "C" int lesbgk_batch_create(int32_t capacity, int32_t nx, void *d_workspa
   for (int w : {1, 2, 4, 8, 16, 32})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(resident_fn(w), cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_range, 0, sizeof(int) * 2 * kNumClasses, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_range, 0, sizeof(int) * 2 * kNumClasses * (1 + kChains), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_range_all, 0, sizeof(int) * 2 * kNumClasses, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_rrange, 0, sizeof(int) * 2 * kBuckets, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1324,7 +1467,7 @@ extern "C" int lesbgk_batch_step(lesbgk_batch *b, int64_t nsteps, void *stream) 
   cudaError_t e = cudaSuccess;
   auto direct_step = [&]() {
     for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls)
-      if (b->range[cls][1]) e = launch_one_step(b, cls, b->par, step_grid(b, b->range[cls][1]), s);
+      if (b->range[cls][1]) e = launch_one_step(b, cls, b->par, s);
     if (e == cudaSuccess) e = launch_resident(b, 1, b->par, b->par ^ 1, s);
     if (e == cudaSuccess) {
       b->par ^= 1;  // the slots' current buffers are desc.f[par]
@@ -1501,7 +1644,7 @@ extern "C" int lesbgk_batch_get_info(const lesbgk_batch *b, int32_t slot, lesbgk
   out->q = (int)stored_values(sl.p);
   out->order = sl.order;
   out->cells_per_thread = 1;
-  out->rows_per_segment = b->rows;
+  out->rows_per_segment = b->auto_rows && b->rows_of[sl.cls] ? b->rows_of[sl.cls] : b->rows;
   return 0;
 }
 
@@ -1511,6 +1654,7 @@ extern "C" int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream
     if (sl.used && (long long)(sl.p.ny + rows - 1) / rows > (long long)kItemsPerSlot)
       return fail(LESBGK_EINVAL, "rows %d too short for ny %d", rows, sl.p.ny);
   b->rows = rows;
+  b->auto_rows = false;
   drop_graph(b);
   return rebuild_items(b, static_cast<cudaStream_t>(stream));
 }
@@ -1523,6 +1667,7 @@ extern "C" int lesbgk_batch_set_resident(lesbgk_batch *b, int32_t on, int32_t st
   if (steps_per_launch && (steps_per_launch < 2 || steps_per_launch > kGraphSteps || (steps_per_launch & 1) ||
                            kGraphSteps % steps_per_launch))
     return fail(LESBGK_EINVAL, "steps per resident launch must be an even divisor of %d", kGraphSteps);
+  b->auto_resident = false;
   b->resident = on != 0;
   if (steps_per_launch) b->resident_k = steps_per_launch;
   drop_graph(b);
@@ -1532,7 +1677,11 @@ extern "C" int lesbgk_batch_set_resident(lesbgk_batch *b, int32_t on, int32_t st
 extern "C" int lesbgk_batch_get_launch(const lesbgk_batch *b, int32_t *rows, int32_t *resident,
                                        int32_t *steps_per_launch, int32_t *resident_max_ny) {
   if (!b) return fail(LESBGK_EINVAL, "batch is NULL");
-  if (rows) *rows = b->rows;
+  if (rows) {
+    *rows = b->rows;
+    for (int cls = kNumClasses - 1; b->auto_rows && cls >= 0; --cls)  // the first class in use
+      if (b->range_all[cls][1] && b->rows_of[cls]) *rows = b->rows_of[cls];
+  }
   if (resident) *resident = b->resident ? 1 : 0;
   if (steps_per_launch) *steps_per_launch = b->resident_k;
   if (resident_max_ny) *resident_max_ny = std::min(b->resident_ny, b->resident_limit);
@@ -1544,17 +1693,19 @@ extern "C" int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates,
   lesbgk_internal::Range range_("lesbgk_batch_autotune");
   if (!b || !candidates || n < 1) return fail(LESBGK_EINVAL, "bad autotune arguments");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaStream_t s2 = nullptr;
+  cudaStream_t s2 = nullptr, sc[kChains - 1] = {};  // resident launches; chains past the first
   cudaEvent_t t0, t1, fork, join;
   cudaError_t e = cudaEventCreate(&t0);
   if (e == cudaSuccess) e = cudaEventCreate(&t1);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking);
+  for (cudaStream_t &x : sc)
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
   if (e != cudaSuccess) return cuda_fail(e, "autotune set-up");
   // candidates: rows per work item x {per-step kernel for all, resident
   // kernel with 16 or 64 steps per launch}; each timed as a 64-step chunk,
-  // the resident launches on a second stream beside the per-step chain (as in
+  // the chains and the resident launches on streams beside one another (as in
   // the graph), every launch reading the current buffers and writing the
   // spare ones, so the state is left untouched
   struct Cand { int rows, res, k, limit; };
@@ -1564,6 +1715,7 @@ extern "C" int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates,
     for (int lim : {64, 128, 256, 1 << 30})
       for (int k : {16, 64}) cands.push_back({candidates[c], 1, k, lim});
   }
+  b->auto_resident = false;
   Cand best{b->rows, b->resident ? 1 : 0, b->resident_k, b->resident_limit};
   float best_ms = 1e30f;
   int rc = 0;
@@ -1577,12 +1729,19 @@ extern "C" int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates,
       e = cudaEventRecord(t0, s);
       if (e == cudaSuccess) e = cudaEventRecord(fork, s);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s2, fork, 0);
+      for (cudaStream_t x : sc)
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(x, fork, 0);
       for (int c = 0; c < kGraphSteps / cd.k && e == cudaSuccess; ++c) e = launch_resident(b, cd.k, b->par, b->par ^ 1, s2);
       if (e == cudaSuccess) e = cudaEventRecord(join, s2);
       for (int st = 0; st < kGraphSteps && e == cudaSuccess; ++st)
         for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls)
-          if (b->range[cls][1]) e = launch_one_step(b, cls, b->par, step_grid(b, b->range[cls][1]), s);
+          for (int c = 0; c < kChains && e == cudaSuccess; ++c)
+            if (b->range_chain[cls][c][1]) e = launch_one_step(b, cls, b->par, c ? sc[c - 1] : s, c);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join, 0);
+      for (cudaStream_t x : sc) {
+        if (e == cudaSuccess) e = cudaEventRecord(join, x);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join, 0);
+      }
       if (e == cudaSuccess) e = cudaEventRecord(t1, s);
       if (e == cudaSuccess) e = cudaEventSynchronize(t1);
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
@@ -1598,6 +1757,7 @@ extern "C" int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates,
   cudaEventDestroy(fork);
   cudaEventDestroy(join);
   cudaStreamDestroy(s2);
+  for (cudaStream_t x : sc) cudaStreamDestroy(x);
   if (rc) return rc;
   if (e != cudaSuccess) return cuda_fail(e, "autotune");
   b->resident = best.res != 0;

@@ -79,3 +79,44 @@ def test_steps_overlap_safely_on_a_busy_stream_and_in_a_graph(nroots, dim, stora
         g.replay()
     torch.cuda.synchronize()
     assert torch.equal(many.populations(), graphed.populations())
+
+
+@pytest.mark.parametrize("nx,n,ny_lo,ny_hi,nroots,dim", [
+    (4, 5, 2, 60, 4, 2),        # short solves only: the resident kernel
+    (4, 40, 2, 300, 4, 2),      # one chain of one-row items
+    (4, 150, 16, 1024, 4, 2),   # around a full chip: several chains
+    (4, 100, 16, 512, 6, 2),
+    (16, 40, 16, 700, 4, 3),
+    (1, 300, 16, 500, 4, 2),
+])
+def test_batch_defaults_give_the_bits_of_fixed_rows(nx, n, ny_lo, ny_hi, nroots, dim):
+    """Rows, chains and the resident kernel as the batch's contents choose
+    them, through step graphs, single steps, removals and re-admissions,
+    against fixed 32-row items without the resident kernel."""
+    import torch
+    from dataclasses import replace
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    probs = [replace(p, nx=nx, nroots=nroots, dim=dim, scheme=I.SPLIT if k % 3 == 0 else I.UNSPLIT)
+             for k, p in enumerate(I.batch_mix(n=n, seed=n, ny_lo=ny_lo, ny_hi=ny_hi))]
+    params = [L.params_from_problem(p) for p in probs]
+    got = []
+    for fixed in (False, True):
+        bt = L.Batch(capacity=n, nx=nx, pool_bytes=sum(L.batch_slot_bytes(p) for p in params) + (1 << 20))
+        if fixed:
+            bt.set_resident(False)
+            bt.set_rows(32)
+        slots = bt.add_many(params)
+        bt.step(64 * 2 + 3)
+        for k in range(0, n, 3):
+            bt.remove(slots[k])
+        bt.step(64)
+        for k in range(0, n, 6):
+            slots[k] = bt.add(params[k])
+        bt.step(70)
+        keep = [k for k in range(n) if k % 3 or k % 6 == 0]
+        got.append([bt.populations(slots[k]) for k in keep])
+        assert int(bt.check_guards().sum()) == 0
+        bt.close()
+    for a, b in zip(*got):
+        assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
