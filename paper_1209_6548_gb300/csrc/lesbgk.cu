@@ -1051,6 +1051,204 @@ __global__ void k_reduce_partials(const double *__restrict__ partial, int n, dou
   if (lane == 0) sums[q] = t;
 }
 
+// ---------------------------------------------------------------------------
+// Many steps of a small solve in one launch (FP32, nx <= 32 periodic columns,
+// steady walls): the whole state stays in the shared memory of one cluster.
+// CTA r owns a band of rows and holds it, with two ghost rows on either side,
+// in two buffers; a thread updates one node per step from five rows of its
+// column, rebuilding the y-stencil that k_step carries by the same operations
+// and then running the same flux, collision and wall code, so the result is
+// bitwise that of k_step.  The x-neighbours are lanes of the same warp (32/nx
+// rows per warp).  A new row near a band's edge also goes to the neighbour's
+// ghost rows through distributed shared memory, a wall row to its own ghost
+// rows; one barrier per step (cluster-wide if there are several CTAs) then
+// swaps the buffers.
+// What bounds it: the latency of one node's chain, 0.7 us (D2Q16) or 1.7 us
+// (D2Q36), and 0.2 us for the cluster's barrier, while no scheduler has two
+// warps.  us per step over 512 steps, k_step -> this kernel: 4x64 D2Q16 2.70 ->
+// 0.94, D2Q36 4.1 -> 1.9, D3Q64 3.5 -> 1.5; 4x1000 D2Q16 3.0 -> 1.24; 32x64
+// D2Q16 2.7 -> 1.24; in a call of three steps 5.6 -> 4.2.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// address of this CTA's shared location `a` in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned cluster_map(unsigned a, unsigned rank) {
+  unsigned r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_store(unsigned addr, uint4 v) {
+  asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_store(unsigned addr, uint2 v) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// neighbour lanes inside a group of nx lanes (periodic in x)
+struct RowLanes {
+  int l, r;
+  __device__ __forceinline__ float left(float v) const { return __shfl_sync(kFull, v, l); }
+  __device__ __forceinline__ float right(float v) const { return __shfl_sync(kFull, v, r); }
+};
+
+// rows [band_start(c), band_start(c + 1)) belong to CTA c of `ctas`
+__host__ __device__ inline int band_start(int ny, int ctas, int c) { return (int)((long long)ny * c / ctas); }
+
+template <int NR, int N, bool SPLIT, int NZ>
+__global__ void __launch_bounds__(NR == 4 && NZ == 1 ? 512 : 256, 1)
+    k_steps_small(float *__restrict__ f, int nsteps, int ctas, const KArgs A) {
+  using Lay = Layout<NR, float, NZ>;
+  using T = typename Raw<Lay::VB>::T;
+  constexpr int Q = Lay::Q, H = Lay::H, V = Lay::V, G = Lay::G;
+  const int nx = A.nx, ny = A.ny;
+  const int rank = ctas > 1 ? (int)cluster_rank() : 0;
+  const int a0 = band_start(ny, ctas, rank), b0 = band_start(ny, ctas, rank + 1);
+  const int most = (ny + ctas - 1) / ctas;  // rows of the largest band
+  const int slots = (most + 4) * nx;        // nodes of a group plane: row slot s holds row a0 - 2 + s
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T *buf = reinterpret_cast<T *>(smem_raw);  // [2][G][slots]
+  for (int t = threadIdx.x; t < (b0 - a0 + 4) * nx; t += blockDim.x) {
+    const int j = map_row(a0 - 2 + t / nx, ny, A.walls);
+    const T *p = reinterpret_cast<const T *>(f) + (long long)j * nx + t % nx;
+#pragma unroll
+    for (int g = 0; g < G; ++g) buf[g * slots + t] = __ldcg(p + g * A.plane);
+  }
+  const int lane = threadIdx.x & 31;
+  const int per = 32 / nx;                       // rows a warp takes
+  const int gi = min(lane / nx, per - 1), x = lane % nx;
+  const RowLanes nb{gi * nx + (x ? x - 1 : nx - 1), gi * nx + (x + 1 < nx ? x + 1 : 0)};
+  const int row = a0 + (int)(threadIdx.x >> 5) * per + gi;
+  const bool live = lane < per * nx && row < b0;
+  const int j = min(row, b0 - 1);  // a spare lane computes a real row and stores nothing
+  const int me = (j - a0 + 2) * nx + x;
+  // where else the new row goes: the neighbours' ghost rows (rows within two of
+  // the band's edges), or this CTA's own at a wall
+  unsigned extra[2] = {0u, 0u};  // shared::cluster addresses in buffer 0, group 0
+  {
+    const unsigned base = static_cast<unsigned>(__cvta_generic_to_shared(buf));
+    auto at = [&](int r, int slot) {
+      const unsigned local = base + (unsigned)((slot * nx + x) * sizeof(T));
+      return cluster_map(local, (unsigned)r);
+    };
+    const bool wlow = A.walls && rank == 0, whigh = A.walls && rank == ctas - 1;
+    if (wlow && j == 0) {
+      extra[0] = at(rank, 0);
+      extra[1] = at(rank, 1);
+    } else if (!wlow && j - a0 < 2) {
+      const int c = rank ? rank - 1 : ctas - 1;
+      extra[0] = at(c, band_start(ny, ctas, c + 1) - band_start(ny, ctas, c) + 2 + j - a0);
+    }
+    if (whigh && j == ny - 1) {
+      extra[0] = at(rank, b0 - a0 + 2);
+      extra[1] = at(rank, b0 - a0 + 3);
+    } else if (!whigh && b0 - j <= 2) {
+      extra[1] = at(rank + 1 < ctas ? rank + 1 : 0, 2 - (b0 - j));
+    }
+  }
+  auto sync = [&] {
+    if (ctas > 1) cluster_barrier();
+    else __syncthreads();
+  };
+  sync();
+  int cur = 0;
+  for (int step = 0; step < nsteps; ++step) {
+    const T *in = buf + (size_t)cur * G * slots + me;
+    float fc[Q], s0[Q], s1[Q], ld[Q];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const T *p = in + g * slots;
+      float m2[Q], m1[Q], p1[Q];
+      unpack_group<NR, float>(p[-nx], g, m1, A);
+      unpack_group<NR, float>(p[0], g, fc, A);
+      unpack_group<NR, float>(p[nx], g, p1, A);
+      if (g >= G / 2) unpack_group<NR, float>(p[-2 * nx], g, m2, A);
+      else unpack_group<NR, float>(p[2 * nx], g, ld, A);
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        const int a = Lay::alpha(g * V + k);
+        if (g >= G / 2) {  // c_y > 0: s0 = f_j - f_{j-1}, s1 = sigma_{j-1}, incoming f_{j+1}
+          s0[a] = fc[a] - m1[a];
+          s1[a] = minmod(m1[a] - m2[a], fc[a] - m1[a]);
+          ld[a] = p1[a];
+        } else {  // c_y < 0: s0 = f_{j+1}, s1 = sigma_j, incoming f_{j+2}
+          s0[a] = p1[a];
+          s1[a] = minmod(fc[a] - m1[a], p1[a] - fc[a]);
+        }
+      }
+    }
+    float acc[Q], xs[Q], omw;
+    collide_any<NR, N>(fc, acc, omw, A, A);
+    const float2 omw2 = make_float2(omw, omw);
+#pragma unroll
+    for (int a = 0; a < Q; a += 2) {
+      const int iy = a % NR;
+      if ((iy >= H) != (iy + 1 >= H)) {  // a pair across c_y = 0 (D2Q36): one at a time
+#pragma unroll
+        for (int b = a; b < a + 2; ++b) {
+          float f0;
+          const float diff = yflux(b % NR >= H, b, fc, s0, s1, ld, A.ky[b % NR], f0);
+          acc[b] = fmaf(omw, f0, fmaf(-A.ay[b % NR], diff, acc[b]));
+          xs[b] = SPLIT ? fmaf(-A.ay[b % NR], diff, f0) : f0;
+        }
+        continue;
+      }
+      const float2 nay = make_float2(A.nay[iy], A.nay[iy + 1]);
+      float2 f0;
+      const float2 diff = yflux2(iy >= H, a, fc, s0, s1, ld, make_float2(A.ky[iy], A.ky[iy + 1]), f0);
+      const float2 ac = fma2(omw2, f0, fma2(nay, diff, make_float2(acc[a], acc[a + 1])));
+      const float2 x2 = SPLIT ? fma2(nay, diff, f0) : f0;
+      acc[a] = ac.x;
+      acc[a + 1] = ac.y;
+      xs[a] = x2.x;
+      xs[a + 1] = x2.y;
+    }
+#pragma unroll
+    for (int a = 0; a < Q; a += 2) {
+      const int ix = (a / NR) % NR;
+      const float2 kx = make_float2(A.kx2[ix][0], A.kx2[ix][1]);
+      const float2 nax = make_float2(A.nax2[ix][0], A.nax2[ix][1]);
+      const float2 diff = xflux2(ix >= H, make_float2(xs[a], xs[a + 1]), kx, nb);
+      const float2 ac = fma2(nax, diff, make_float2(acc[a], acc[a + 1]));
+      acc[a] = ac.x;
+      acc[a + 1] = ac.y;
+    }
+    if (A.walls && (j == 0 || j == ny - 1)) {
+      if (A.wspec != 0.0f) wall_fix<NR, true>(acc, j == 0 ? 0 : 1, A, A);
+      else wall_fix<NR, false>(acc, j == 0 ? 0 : 1, A, A);
+    }
+    cur ^= 1;
+    if (live) {
+      const unsigned shift = (unsigned)(cur * G * slots * (int)sizeof(T));
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        T raw;
+        float *e = reinterpret_cast<float *>(&raw);
+#pragma unroll
+        for (int k = 0; k < V; ++k) e[k] = acc[Lay::alpha(g * V + k)];
+        buf[(size_t)cur * G * slots + g * slots + me] = raw;
+        const unsigned off = shift + (unsigned)(g * slots * (int)sizeof(T));
+        if (extra[0]) cluster_store(extra[0] + off, raw);
+        if (extra[1]) cluster_store(extra[1] + off, raw);
+      }
+    }
+    sync();
+  }
+  // (every CTA is past its last remote store: the barrier above)
+  if (live) {
+    T *p = reinterpret_cast<T *>(f) + (long long)j * nx + x;
+    const T *in = buf + (size_t)cur * G * slots + me;
+#pragma unroll
+    for (int g = 0; g < G; ++g) p[g * A.plane] = in[g * slots];
+  }
+}
+
 constexpr int kMomGrid = lesbgk_internal::kMomentPartials;
 
 }  // namespace
@@ -1072,6 +1270,8 @@ struct lesbgk {
   double dt, dx, dy, cmax, tau_ref;
   int64_t steps;
   int sm_count;
+  bool rows_set;   // rows per segment chosen by the caller: every step takes that kernel
+  int small_ctas;  // cluster size of k_steps_small, 0 where the solve does not fit it
 };
 
 namespace {
@@ -1322,6 +1522,97 @@ int launch_step(lesbgk *h, const void *fin, void *fout, cudaStream_t s) {
   return 0;
 }
 
+int small_warps(const lesbgk *h, int ctas) {  // warps of the largest band
+  const int per = 32 / h->p.nx, most = (h->p.ny + ctas - 1) / ctas;
+  return (most + per - 1) / per;
+}
+
+constexpr int kSmallSmem = 200 * 1024;
+size_t small_smem(const lesbgk *h, int ctas) {  // two buffers of Q planes with four ghost rows
+  const int most = (h->p.ny + ctas - 1) / ctas;
+  return (size_t)2 * h->q * sizeof(float) * (most + 4) * h->p.nx;
+}
+
+// fn(kernel) for the handle's set and scheme.
+template <class Fn>
+void with_small(const lesbgk *h, Fn &&fn) {
+  const bool split = h->p.scheme == LESBGK_SPLIT;
+  if (h->nr == 6) split ? fn(k_steps_small<6, 4, true, 1>) : fn(k_steps_small<6, 4, false, 1>);
+  else if (h->q == 32) split ? fn(k_steps_small<4, 3, true, 2>) : fn(k_steps_small<4, 3, false, 2>);
+  else split ? fn(k_steps_small<4, 3, true, 1>) : fn(k_steps_small<4, 3, false, 1>);
+}
+
+cudaLaunchAttribute cluster_of(int ctas) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ctas;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  return at;
+}
+
+cudaLaunchConfig_t small_config(const lesbgk *h, int ctas) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(ctas);
+  c.blockDim = dim3(32 * small_warps(h, ctas));
+  c.dynamicSmemBytes = small_smem(h, ctas);
+  return c;
+}
+
+// The cluster size for k_steps_small, or 0: FP32 solves of few periodic columns
+// with steady walls whose rows fit its CTAs at one node per thread.  A step
+// takes one warp's latency while no scheduler has a second warp, half of it
+// more for each further one, and a quarter more for the cluster's barrier
+// (4x1000 D2Q16, us per step on 2, 4, 8, 16 CTAs: too tall, too tall, 1.97, 1.24;
+// 4x64: 0.94, 0.88, 0.93, 0.92, on one 1.09).
+int pick_small(const lesbgk *h) {
+  const bool built = (h->nr == 4 && h->order == 3 && h->q <= 32) || (h->nr == 6 && h->order == 4 && h->q == 36);
+  if (!built || h->p.storage != LESBGK_F32 || h->p.nx > 32 || h->p.ny < 4 || h->args.xwalls || heated_walls(h->su))
+    return 0;
+  const int most_warps = h->q >= 32 ? 8 : 16;
+  int best = 0;
+  double least = 0.0;
+  for (int c = 1; c <= 16; c *= 2) {
+    const int w = small_warps(h, c);
+    if (w > most_warps || h->p.ny / c < 4 || small_smem(h, c) > (size_t)kSmallSmem) continue;
+    const double t = 0.5 + 0.5 * ((w + 3) / 4) + (c > 1 ? 0.25 : 0.0);
+    if (best && t >= least) continue;
+    if (c > 1) {  // (16 CTAs are past the portable size)
+      cudaLaunchConfig_t cfg = small_config(h, c);
+      cudaLaunchAttribute at = cluster_of(c);
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      with_small(h, [&](auto kernel) {
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) n = 0;
+      });
+      cudaGetLastError();
+      if (n < 1) continue;
+    }
+    best = c;
+    least = t;
+  }
+  return best;
+}
+
+// nsteps steps of a small solve in place, in launches of at most kSmallSteps
+// (a few milliseconds each).
+constexpr int64_t kSmallSteps = 4096, kSmallFrom = 3;
+cudaError_t launch_small(lesbgk *h, int64_t nsteps, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  const int ctas = h->small_ctas;
+  for (int64_t done = 0; done < nsteps && e == cudaSuccess;) {
+    const int n = (int)(nsteps - done < kSmallSteps ? nsteps - done : kSmallSteps);
+    cudaLaunchAttribute at = cluster_of(ctas);
+    cudaLaunchConfig_t c = small_config(h, ctas);
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    with_small(h, [&](auto kernel) { e = cudaLaunchKernelEx(&c, kernel, h->buf[h->cur], n, ctas, h->args); });
+    done += n;
+  }
+  return e;
+}
+
 unsigned grid_for(const lesbgk *h, long long cells) {
   long long g = (cells + kBlock - 1) / kBlock;
   const long long cap = (long long)h->sm_count * 16;
@@ -1466,6 +1757,13 @@ extern "C" int lesbgk_create(const lesbgk_params *p, void *d_workspace, size_t b
   }
   pick_launch(h);
   e = allow_smem(h);
+  if (e == cudaSuccess && p->storage == LESBGK_F32 && p->nx <= 32) {
+    with_small(h, [&](auto kernel) {
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmem);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    });
+    if (e == cudaSuccess) h->small_ctas = pick_small(h);
+  }
   if (e != cudaSuccess) {
     delete h;
     return cuda_fail(e, "step kernel shared-memory opt-in");
@@ -1496,6 +1794,12 @@ extern "C" int lesbgk_step(lesbgk *h, int64_t nsteps, void *stream) {
   if (!h) return fail(LESBGK_EINVAL, "handle is NULL");
   if (nsteps < 0) return fail(LESBGK_EINVAL, "nsteps < 0");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (h->small_ctas && !h->rows_set && nsteps >= kSmallFrom) {
+    cudaError_t e = launch_small(h, nsteps, s);
+    if (e != cudaSuccess) return cuda_fail(e, "step kernel");
+    h->steps += nsteps;
+    return 0;
+  }
   for (int64_t k = 0; k < nsteps; ++k) {
     h->args.seed = (unsigned)(h->steps + k) * 0x9e3779b9u + 0x7f4a7c15u;  // a new rounding key per step
     if (heated_walls(h->su))  // wall tables at the time of the state written
@@ -1690,7 +1994,10 @@ extern "C" int lesbgk_set_launch(lesbgk *h, int32_t cells_per_thread, int32_t ro
   if (!h) return fail(LESBGK_EINVAL, "handle is NULL");
   if (cells_per_thread < 0 || cells_per_thread > 1 || rows_per_segment < 0)
     return fail(LESBGK_EINVAL, "bad launch shape (cells_per_thread must be 0 or 1)");
-  if (rows_per_segment) h->rows = rows_per_segment;
+  if (rows_per_segment) {
+    h->rows = rows_per_segment;
+    h->rows_set = true;
+  }
   return pick_launch(h);
 }
 

@@ -120,3 +120,54 @@ def test_batch_defaults_give_the_bits_of_fixed_rows(nx, n, ny_lo, ny_hi, nroots,
         bt.close()
     for a, b in zip(*got):
         assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nx,ny", [(4, 64), (1, 4), (2, 5), (3, 33), (4, 1024), (5, 200), (7, 65), (31, 24), (32, 128),
+                                   (16, 131), (33, 20), (4, 3)])
+@pytest.mark.parametrize("nroots,dim", [(4, 2), (6, 2), (4, 3)])
+def test_small_solves_stay_on_chip_with_the_bits_of_single_steps(nx, ny, nroots, dim):
+    """Calls of several steps on few columns keep the state in a cluster's
+    shared memory; single-step calls and fixed rows take the marching kernel.
+    Band edges, ghost rows (periodic, wall), spare lanes, columns that do not
+    divide a warp, and sizes just outside the range."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    for bc_y, scheme, spec in ((I.DIFFUSE, I.UNSPLIT, 0.0), (I.DIFFUSE, I.SPLIT, 0.4), (I.PERIODIC, I.SPLIT, 0.0),
+                               (I.PERIODIC, I.UNSPLIT, 0.0)):
+        prob = I.Problem(name="small", nroots=nroots, dim=dim, nx=nx, ny=ny, bc_y=bc_y, kn=0.1, b=-0.5, scheme=scheme,
+                         wall_ux=(-0.05, 0.05), wall_T=(0.97, 1.02), wall_specular=spec, g=(1e-3, 2e-4))
+        p = L.params_from_problem(prob)
+        init = I.random_fields(prob, amp_u=0.02, amp_T=0.02, amp_rho=0.02, seed=ny)
+        got = []
+        for mode in ("calls", "single", "rows"):
+            s = L.Solver(p, h_init=init)
+            if mode == "rows":
+                s.set_launch(0, 3)
+            if mode == "single":
+                for _ in range(11):
+                    s.step(1)
+            else:
+                for n in (3, 1, 5, 2):
+                    s.step(n)
+            assert s.info.steps_done == 11
+            got.append(s.populations())
+        assert bool(torch.isfinite(got[0]).all())
+        assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
+
+
+def test_small_solves_run_past_one_launch_of_steps():
+    """More steps than one launch takes (4096), on a stream of its own."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    p = L.params_from_problem(I.couette_4x64())
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        a, b = L.Solver(p, stream=side), L.Solver(p, stream=side)
+        a.step(4096 + 100)
+        b.set_launch(0, 4)
+        b.step(4096 + 100)
+        same = torch.equal(a.populations(), b.populations())
+    side.synchronize()
+    assert same
