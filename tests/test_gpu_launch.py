@@ -171,3 +171,36 @@ def test_small_solves_run_past_one_launch_of_steps():
         same = torch.equal(a.populations(), b.populations())
     side.synchronize()
     assert same
+
+
+@pytest.mark.parametrize("capacity,count,ny_hi", [(2, 2, 90), (70, 70, 700), (40, 23, 65), (300, 300, 1024)])
+def test_fields_of_many_admissions_arrive_whole(capacity, count, ny_hi):
+    """Fields staged in pieces, in slot and class order of their own, larger
+    than the staging area (which grows with the capacity), absent for some:
+    the populations of single admissions, bitwise."""
+    import torch
+    from dataclasses import replace
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    probs = [replace(p, nroots=6 if k % 4 == 1 else 4, dim=3 if k % 4 == 2 else 2)
+             for k, p in enumerate(I.batch_mix(n=count, seed=count, ny_lo=16, ny_hi=ny_hi))]
+    if capacity == 2:
+        probs[0] = replace(probs[0], ny=1500)  # 192 kB of fields: more than two slots' staging
+    params = [L.params_from_problem(p) for p in probs]
+    for k, p in enumerate(params):
+        p.storage = (0, 1, 2)[k % 3]
+    fields = [None if k % 5 == 3 else I.random_fields(p, seed=k) for k, p in enumerate(probs)]
+    pool = sum(L.batch_slot_bytes(p) for p in params)
+    many = L.Batch(capacity=capacity, nx=4, pool_bytes=pool)
+    slots = many.add_many(params, fields)
+    one = L.Batch(capacity=capacity, nx=4, pool_bytes=pool)
+    for s, p, f in zip(slots, params, fields):
+        assert torch.equal(many.populations(s), one.populations(one.add(p, f)))
+    assert int(many.check_guards().sum()) == 0
+    bad = [f.copy() if f is not None else None for f in fields]
+    bad[0][3, 1, 2] = np.nan
+    three = L.Batch(capacity=capacity, nx=4, pool_bytes=pool)
+    with pytest.raises(L.LesbgkError) as err:
+        three.add_many(params, bad)
+    assert "node 6 " in str(err.value)
+    assert three.pool_free()[1] >= pool  # nothing was kept
