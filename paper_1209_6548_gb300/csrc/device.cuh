@@ -784,17 +784,6 @@ struct Raw<8> { using T = uint2; };
 template <>
 struct Raw<4> { using T = unsigned; };
 
-// Load group g of one node (p points at the node's row, group 0) into F[alpha].
-template <int NR, int Q>
-__device__ __forceinline__ void ld_group(const float *p, long long gstride, int g, float (&F)[Q]) {
-  using L = LayoutQ<NR, float, Q>;
-  using T = typename VecT<L::V>::T;
-  const T v = __ldg(reinterpret_cast<const T *>(p + g * gstride));
-  const float *e = reinterpret_cast<const float *>(&v);
-#pragma unroll
-  for (int k = 0; k < L::V; ++k) F[L::alpha(g * L::V + k)] = e[k];
-}
-
 template <int NR, int Q>
 __device__ __forceinline__ void st_group(float *p, long long gstride, int g, const float (&F)[Q]) {
   using L = LayoutQ<NR, float, Q>;
@@ -820,15 +809,9 @@ __device__ __forceinline__ void unpack_group(const typename Raw<LayoutQ<NR, S, Q
   }
 }
 
-template <int NR, class S, int Q, class TT>
-__device__ __forceinline__ void ld_group_s(const S *p, long long gstride, int g, float (&F)[Q], const TT &Tt) {
-  using R = typename Raw<LayoutQ<NR, S, Q>::VB>::T;
-  const R raw = __ldg(reinterpret_cast<const R *>(p + g * gstride));
-  unpack_group<NR, S>(raw, g, F, Tt);
-}
-
-// The same past L1 (and never through the read-only path): for buffers that
-// the previous kernel may still have been writing when this one started.
+// Load group g of one node (p points at the node's row, group 0) into F[alpha];
+// past L1 and never through the read-only path: the previous kernel may still
+// have been writing the buffer when this one started.
 template <int NR, class S, int Q, class TT>
 __device__ __forceinline__ void ld_group_cg(const S *p, long long gstride, int g, float (&F)[Q], const TT &Tt) {
   using R = typename Raw<LayoutQ<NR, S, Q>::VB>::T;
@@ -912,7 +895,8 @@ __device__ __forceinline__ __half *lo_plane(float *f, long long plane) {
 }
 
 // All stored values of node c as FP32 deviations (for Comp, hi + lo rounded
-// once); f at the grid's (or a row's) start, plane = nx ny.
+// once); f at the grid's (or a row's) start, plane = nx ny.  Past L1: read once,
+// and the kernel may have started while the previous one still wrote.
 template <int NR, class S, int NZ, class TT>
 __device__ __forceinline__ void ld_node(const typename Elem<S>::T *f, long long c, long long plane,
                                         float (&F)[NZ * NR * NR], const TT &Tt) {
@@ -921,11 +905,11 @@ __device__ __forceinline__ void ld_node(const typename Elem<S>::T *f, long long 
     using LL = Layout<NR, __half, NZ>;
     static_assert(LL::V == 2 * LH::V, "hi and lo vectors of 16 bytes");
 #pragma unroll
-    for (int g = 0; g < LH::G; ++g) ld_group<NR>(f + c * LH::V, (long long)LH::V * plane, g, F);
+    for (int g = 0; g < LH::G; ++g) ld_group_cg<NR, float>(f + c * LH::V, (long long)LH::V * plane, g, F, Tt);
     const __half *lo = lo_plane<LH::Q>(f, plane) + c * LL::V;
 #pragma unroll
     for (int g = 0; g < LL::G; ++g) {
-      const uint4 raw = __ldg(reinterpret_cast<const uint4 *>(lo + (long long)g * LL::V * plane));
+      const uint4 raw = __ldcg(reinterpret_cast<const uint4 *>(lo + (long long)g * LL::V * plane));
       const __half *e = reinterpret_cast<const __half *>(&raw);
 #pragma unroll
       for (int k = 0; k < LL::V; ++k) {
@@ -936,11 +920,11 @@ __device__ __forceinline__ void ld_node(const typename Elem<S>::T *f, long long 
   } else if constexpr (std::is_same<S, float>::value) {  // (no scale tables needed)
     using L = Layout<NR, float, NZ>;
 #pragma unroll
-    for (int g = 0; g < L::G; ++g) ld_group<NR>(f + c * L::V, (long long)L::V * plane, g, F);
+    for (int g = 0; g < L::G; ++g) ld_group_cg<NR, float>(f + c * L::V, (long long)L::V * plane, g, F, Tt);
   } else {
     using L = Layout<NR, S, NZ>;
 #pragma unroll
-    for (int g = 0; g < L::G; ++g) ld_group_s<NR, S>(f + c * L::V, (long long)L::V * plane, g, F, Tt);
+    for (int g = 0; g < L::G; ++g) ld_group_cg<NR, S>(f + c * L::V, (long long)L::V * plane, g, F, Tt);
   }
 }
 

@@ -811,15 +811,17 @@ __global__ void __launch_bounds__(kBlock, NZ == 1 ? 3 : 1) k_step_c(const float 
 template <int NR, int N, class S, int NZ = 1>
 __global__ void __launch_bounds__(kBlock) k_init(const double *__restrict__ fields,
                                                  typename Elem<S>::T *__restrict__ f, const KArgs A) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int Q = NZ * NR * NR;
   const long long cells = A.plane;
   for (long long c = blockIdx.x * (long long)kBlock + threadIdx.x; c < cells; c += (long long)gridDim.x * kBlock) {
     float drho = 0.f, ux = 0.f, uy = 0.f, dT = 0.f;
     if (fields) {
-      drho = (float)(fields[c] - 1.0);
-      ux = (float)fields[cells + c];
-      uy = (float)fields[2 * cells + c];
-      dT = (float)(fields[3 * cells + c] - 1.0);
+      drho = (float)(__ldcg(fields + c) - 1.0);
+      ux = (float)__ldcg(fields + cells + c);
+      uy = (float)__ldcg(fields + 2 * cells + c);
+      dT = (float)(__ldcg(fields + 3 * cells + c) - 1.0);
     }
     const float rho = 1.0f + drho;
     const float rdT = rho * dT;
@@ -877,6 +879,8 @@ __global__ void __launch_bounds__(kBlock) k_field_stats(const double *__restrict
 template <int NR, class S, int NZ = 1>
 __global__ void __launch_bounds__(kBlock) k_ungroup(const typename Elem<S>::T *__restrict__ f,
                                                     float *__restrict__ out, long long cells, const KArgs A) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int Q = NZ * NR * NR;
   for (long long c = blockIdx.x * (long long)kBlock + threadIdx.x; c < cells; c += (long long)gridDim.x * kBlock) {
     float F[Q];
@@ -889,11 +893,13 @@ __global__ void __launch_bounds__(kBlock) k_ungroup(const typename Elem<S>::T *_
 template <int NR, class S, int NZ = 1>
 __global__ void __launch_bounds__(kBlock) k_group(const float *__restrict__ in, typename Elem<S>::T *__restrict__ f,
                                                   long long cells, const KArgs A) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int Q = NZ * NR * NR;
   for (long long c = blockIdx.x * (long long)kBlock + threadIdx.x; c < cells; c += (long long)gridDim.x * kBlock) {
     float F[Q];
 #pragma unroll
-    for (int a = 0; a < Q; ++a) F[a] = __ldg(in + a * cells + c);
+    for (int a = 0; a < Q; ++a) F[a] = __ldcg(in + a * cells + c);
     st_node<NR, S, NZ>(f, c, cells, F, A);
   }
 }
@@ -954,6 +960,8 @@ template <int NR, class S, int NZ = 1>
 __global__ void __launch_bounds__(kMomBlock) k_moments(const typename Elem<S>::T *__restrict__ f,
                                                        float *__restrict__ out, double *__restrict__ partial,
                                                        long long cells, long long plane, const KArgs A) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int Q = NZ * NR * NR;
   ConsSums cs;
   for (long long c = blockIdx.x * (long long)kMomBlock + threadIdx.x; c < cells;
@@ -977,6 +985,8 @@ __global__ void __launch_bounds__(kMomBlock) k_residual(const typename Elem<S>::
                                                         float *__restrict__ snap, int update_only,
                                                         unsigned *__restrict__ rbits, double *__restrict__ mpart,
                                                         const KArgs A) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int Q = NZ * NR * NR;
   const long long cells = A.plane;
   float rmax = 0.0f, dm = 0.0f;
@@ -1031,21 +1041,25 @@ __global__ void __launch_bounds__(kMomBlock) k_residual(const typename Elem<S>::
 
 // Sum of n doubles in a fixed order (one warp): bitwise reproducible.
 __global__ void k_reduce_one(const double *__restrict__ part, int n, double *__restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   if (threadIdx.x >= 32) return;
   double t = 0.0;
-  for (int k = lane; k < n; k += 32) t += part[k];
+  for (int k = lane; k < n; k += 32) t += __ldcg(part + k);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(kFull, t, o);
   if (lane == 0) *out = t;
 }
 
 __global__ void k_reduce_partials(const double *__restrict__ partial, int n, double *__restrict__ sums) {
+  pdl_wait();
+  pdl_trigger();
   // one warp per quantity, fixed order: bitwise reproducible
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (q >= 4) return;
   double t = 0.0;
-  for (int k = lane; k < n; k += 32) t += partial[k * 4 + q];
+  for (int k = lane; k < n; k += 32) t += __ldcg(partial + k * 4 + q);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(kFull, t, o);
   if (lane == 0) sums[q] = t;
@@ -1114,6 +1128,8 @@ __global__ void __launch_bounds__(NR == 4 && NZ == 1 ? 512 : 256, 1)
   const int slots = (most + 4) * nx;        // nodes of a group plane: row slot s holds row a0 - 2 + s
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *buf = reinterpret_cast<T *>(smem_raw);  // [2][G][slots]
+  pdl_wait();
+  pdl_trigger();
   for (int t = threadIdx.x; t < (b0 - a0 + 4) * nx; t += blockDim.x) {
     const int j = map_row(a0 - 2 + t / nx, ny, A.walls);
     const T *p = reinterpret_cast<const T *>(f) + (long long)j * nx + t % nx;
@@ -1270,6 +1286,7 @@ struct lesbgk {
   double dt, dx, dy, cmax, tau_ref;
   int64_t steps;
   int sm_count;
+  bool fills;      // a step's blocks take (nearly) every slot of the chip
   bool rows_set;   // rows per segment chosen by the caller: every step takes that kernel
   int small_ctas;  // cluster size of k_steps_small, 0 where the solve does not fit it
 };
@@ -1277,6 +1294,24 @@ struct lesbgk {
 namespace {
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// Launch a kernel that waits for its predecessors itself (pdl_wait before its
+// first access): the launch then overlaps the previous kernel's end.  A solve
+// of 64 steps on 4x64, its moments and its state are four such launches: 94.2 us
+// a pass before, 69.0 with them (and without totals nobody asked for).
+template <class... P, class... Args>
+void launch_overlapped(void (*kernel)(P...), unsigned blocks, unsigned threads, cudaStream_t s, Args... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(blocks);
+  c.blockDim = dim3(threads);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
 
 size_t buffer_bytes(const lesbgk_params *p) {
   const size_t cells = (size_t)p->nx * p->ny;
@@ -1350,6 +1385,8 @@ int pick_launch(lesbgk *h) {
   h->args.rows = h->rows;
   h->args.nstrips = nstrips;
   h->args.nseg = (ny + h->rows - 1) / h->rows;
+  const double blocks = (double)nstrips * h->args.nseg / (h->q >= 100 ? 1 : kBlock / 32);
+  h->fills = blocks >= (slots - 0.5) * (h->sm_count > 0 ? h->sm_count : 152);
   return 0;
 }
 
@@ -1451,7 +1488,7 @@ cudaError_t allow_smem(const lesbgk *h) {
   return e;
 }
 
-int launch_step(lesbgk *h, const void *fin, void *fout, cudaStream_t s) {
+int launch_step(lesbgk *h, const void *fin, void *fout, bool overlap, cudaStream_t s) {
   const long long warps = (long long)h->args.nstrips * h->args.nseg;
   const unsigned grid = (unsigned)((warps * 32 + kBlock - 1) / kBlock);
   dispatch(h->nr, h->order, h->p.storage, h->p.dim, [&](auto r, auto n, auto st, auto z) {
@@ -1464,11 +1501,11 @@ int launch_step(lesbgk *h, const void *fin, void *fout, cudaStream_t s) {
     // wait for it before their first load): hides the launch and the drain,
     // about 2.5 us of every step (us per step, before -> now: 4x64 4.1 -> 2.7,
     // 256^2 cavity 8.2 -> 5.0, 512x1024 16.4 -> 14.8, 1024^2 31.8 -> 29.1,
-    // 4096^2 356.8 -> 354.3)
+    // 4096^2 356.8 -> 354.3); `overlap` false: the previous kernel ends first
     auto go = [&](auto kernel, unsigned blocks, unsigned threads, size_t smem) {
       cudaLaunchAttribute at{};
       at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      at.val.programmaticStreamSerializationAllowed = 1;
+      at.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
       cudaLaunchConfig_t c{};
       c.gridDim = dim3(blocks);
       c.blockDim = dim3(threads);
@@ -1602,11 +1639,13 @@ cudaError_t launch_small(lesbgk *h, int64_t nsteps, cudaStream_t s) {
   const int ctas = h->small_ctas;
   for (int64_t done = 0; done < nsteps && e == cudaSuccess;) {
     const int n = (int)(nsteps - done < kSmallSteps ? nsteps - done : kSmallSteps);
-    cudaLaunchAttribute at = cluster_of(ctas);
+    cudaLaunchAttribute at[2] = {cluster_of(ctas), {}};
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t c = small_config(h, ctas);
     c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = 1;
+    c.attrs = at;
+    c.numAttrs = 2;
     with_small(h, [&](auto kernel) { e = cudaLaunchKernelEx(&c, kernel, h->buf[h->cur], n, ctas, h->args); });
     done += n;
   }
@@ -1625,20 +1664,30 @@ int launch_init(lesbgk *h, const double *fields, void *f, cudaStream_t s) {
   dispatch(h->nr, h->order, h->p.storage, h->p.dim, [&](auto r, auto n, auto st, auto z) {
     constexpr int NR = decltype(r)::value, N = decltype(n)::value, NZ = decltype(z)::value;
     using S = decltype(st);
-    k_init<NR, N, S, NZ><<<grid, kBlock, 0, s>>>(fields, static_cast<typename Elem<S>::T *>(f), h->args);
+    launch_overlapped(k_init<NR, N, S, NZ>, grid, kBlock, s, fields, static_cast<typename Elem<S>::T *>(f), h->args);
   });
   return 0;
 }
 
-int launch_moments(lesbgk *h, float *out, cudaStream_t s) {
+// Blocks of the moment and residual kernels: one node per thread up to
+// kMomGrid blocks (the nodes of each block, and so the totals, are the same
+// for any larger grid).
+unsigned mom_blocks(long long cells) {
+  const long long g = (cells + kMomBlock - 1) / kMomBlock;
+  return (unsigned)(g < 1 ? 1 : g < kMomGrid ? g : kMomGrid);
+}
+
+// Moments of the current state; the totals to h->sums where asked for.
+int launch_moments(lesbgk *h, float *out, bool totals, cudaStream_t s) {
   const void *f = h->buf[h->cur];
+  const unsigned blocks = mom_blocks(h->args.plane);
   dispatch(h->nr, h->order, h->p.storage, h->p.dim, [&](auto r, auto, auto st, auto z) {
     constexpr int NR = decltype(r)::value, NZ = decltype(z)::value;
     using S = decltype(st);
-    k_moments<NR, S, NZ><<<kMomGrid, kMomBlock, 0, s>>>(static_cast<const typename Elem<S>::T *>(f), out,
-                                                        h->partial, h->args.plane, h->args.plane, h->args);
+    launch_overlapped(k_moments<NR, S, NZ>, blocks, kMomBlock, s, static_cast<const typename Elem<S>::T *>(f), out,
+                      h->partial, h->args.plane, h->args.plane, h->args);
   });
-  k_reduce_partials<<<1, 128, 0, s>>>(h->partial, kMomGrid, h->sums);
+  if (totals) launch_overlapped(k_reduce_partials, 1, 128, s, h->partial, (int)blocks, h->sums);
   return 0;
 }
 
@@ -1656,21 +1705,22 @@ cudaError_t launch_init(const KArgs &A, int nr, int order, int storage, int dim,
   dispatch(nr, order, storage, dim, [&](auto r, auto n, auto st, auto z) {
     using S = decltype(st);
     if constexpr (!kIsComp<S> && decltype(z)::value < 3)
-      k_init<decltype(r)::value, decltype(n)::value, S, decltype(z)::value>
-          <<<grid, kBlock, 0, s>>>(fields, static_cast<S *>(f), A);
+      launch_overlapped(k_init<decltype(r)::value, decltype(n)::value, S, decltype(z)::value>, grid, kBlock, s, fields,
+                        static_cast<S *>(f), A);
   });
   return cudaGetLastError();
 }
 
 cudaError_t launch_moments(const KArgs &A, int nr, int order, int storage, int dim, const void *f, float *out,
                            double *partial, double *sums, cudaStream_t s) {
+  const unsigned blocks = mom_blocks(A.plane);
   dispatch(nr, order, storage, dim, [&](auto r, auto, auto st, auto z) {
     using S = decltype(st);
     if constexpr (!kIsComp<S> && decltype(z)::value < 3)
-      k_moments<decltype(r)::value, S, decltype(z)::value>
-          <<<kMomGrid, kMomBlock, 0, s>>>(static_cast<const S *>(f), out, partial, A.plane, A.plane, A);
+      launch_overlapped(k_moments<decltype(r)::value, S, decltype(z)::value>, blocks, kMomBlock, s,
+                        static_cast<const S *>(f), out, partial, A.plane, A.plane, A);
   });
-  k_reduce_partials<<<1, 128, 0, s>>>(partial, kMomGrid, sums);
+  launch_overlapped(k_reduce_partials, 1, 128, s, partial, (int)blocks, sums);
   return cudaGetLastError();
 }
 
@@ -1682,7 +1732,8 @@ cudaError_t launch_ungroup(const KArgs &A, int nr, int order, int storage, int d
   dispatch(nr, order, storage, dim, [&](auto r, auto, auto st, auto z) {
     using S = decltype(st);
     if constexpr (!kIsComp<S> && decltype(z)::value < 3)
-      k_ungroup<decltype(r)::value, S, decltype(z)::value><<<grid, kBlock, 0, s>>>(static_cast<const S *>(f), out, cells, A);
+      launch_overlapped(k_ungroup<decltype(r)::value, S, decltype(z)::value>, grid, kBlock, s, static_cast<const S *>(f),
+                        out, cells, A);
   });
   return cudaGetLastError();
 }
@@ -1804,7 +1855,12 @@ extern "C" int lesbgk_step(lesbgk *h, int64_t nsteps, void *stream) {
     h->args.seed = (unsigned)(h->steps + k) * 0x9e3779b9u + 0x7f4a7c15u;  // a new rounding key per step
     if (heated_walls(h->su))  // wall tables at the time of the state written
       set_wall_time(h->su, (double)(h->steps + k + 1) * h->dt, &h->args);
-    launch_step(h, h->buf[h->cur], h->buf[h->cur ^ 1], s);
+    // A step's blocks enter the slots that the previous step's leave.  Where
+    // they do not fill the chip, blocks that some other kernel once crowded
+    // onto a part of it would stay crowded step after step (512x1024: 24 us per
+    // step instead of 14.8), so a call, and every 32nd step of it, starts on a
+    // drained stream.
+    launch_step(h, h->buf[h->cur], h->buf[h->cur ^ 1], h->fills || k % 32 != 0, s);
     h->cur ^= 1;
   }
   h->steps += nsteps;
@@ -1829,7 +1885,7 @@ extern "C" int lesbgk_moments(lesbgk *h, float *d_out, double *h_sums, void *str
   lesbgk_internal::Range range_("lesbgk_moments");
   if (!h) return fail(LESBGK_EINVAL, "handle is NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  launch_moments(h, d_out, s);
+  launch_moments(h, d_out, h_sums != nullptr, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "moments kernel");
   return finish_sums(h, h_sums, s);
@@ -1841,7 +1897,7 @@ extern "C" int lesbgk_moments_host(lesbgk *h, float *h_out, double *h_sums, void
   if (!h_out) return fail(LESBGK_EINVAL, "h_out is NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   float *stage = h->buf[h->cur ^ 1];  // the spare ping-pong buffer holds >= 9 floats per node
-  launch_moments(h, stage, s);
+  launch_moments(h, stage, h_sums != nullptr, s);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h_out, stage, (size_t)9 * h->args.plane * sizeof(float), cudaMemcpyDeviceToHost, s);
@@ -1860,16 +1916,18 @@ extern "C" int lesbgk_residual(lesbgk *h, float *d_snap, int64_t steps, double *
   unsigned *rbits = reinterpret_cast<unsigned *>(h->sums);
   cudaError_t e = cudaMemsetAsync(rbits, 0, sizeof(unsigned), s);
   const void *f = h->buf[h->cur];
+  const unsigned blocks = mom_blocks(h->args.plane);
   if (e == cudaSuccess) {
     dispatch(h->nr, h->order, h->p.storage, h->p.dim, [&](auto r, auto, auto st, auto z) {
       using S = decltype(st);
-      k_residual<decltype(r)::value, S, decltype(z)::value><<<kMomGrid, kMomBlock, 0, s>>>(
-          static_cast<const typename Elem<S>::T *>(f), d_snap, steps <= 0 ? 1 : 0, rbits, h->partial, h->args);
+      launch_overlapped(k_residual<decltype(r)::value, S, decltype(z)::value>, blocks, kMomBlock, s,
+                        static_cast<const typename Elem<S>::T *>(f), d_snap, steps <= 0 ? 1 : 0, rbits, h->partial,
+                        h->args);
     });
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    k_reduce_one<<<1, 32, 0, s>>>(h->partial, kMomGrid, h->sums + 1);
+    launch_overlapped(k_reduce_one, 1, 32, s, h->partial, (int)blocks, h->sums + 1);
     e = cudaGetLastError();
   }
   double hb[2] = {0.0, 0.0};
@@ -1890,8 +1948,8 @@ extern "C" int lesbgk_get_populations(lesbgk *h, float *d_out, void *stream) {
   const void *f = h->buf[h->cur];
   dispatch(h->nr, h->order, h->p.storage, h->p.dim, [&](auto r, auto, auto st, auto z) {
     using S = decltype(st);
-    k_ungroup<decltype(r)::value, S, decltype(z)::value>
-        <<<grid_for(h, cells), kBlock, 0, s>>>(static_cast<const typename Elem<S>::T *>(f), d_out, cells, h->args);
+    launch_overlapped(k_ungroup<decltype(r)::value, S, decltype(z)::value>, grid_for(h, cells), kBlock, s,
+                      static_cast<const typename Elem<S>::T *>(f), d_out, cells, h->args);
   });
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 0 : cuda_fail(e, "get populations");
@@ -1904,8 +1962,8 @@ extern "C" int lesbgk_set_populations(lesbgk *h, const float *d_in, int64_t step
   void *f = h->buf[h->cur];
   dispatch(h->nr, h->order, h->p.storage, h->p.dim, [&](auto r, auto, auto st, auto z) {
     using S = decltype(st);
-    k_group<decltype(r)::value, S, decltype(z)::value>
-        <<<grid_for(h, cells), kBlock, 0, s>>>(d_in, static_cast<typename Elem<S>::T *>(f), cells, h->args);
+    launch_overlapped(k_group<decltype(r)::value, S, decltype(z)::value>, grid_for(h, cells), kBlock, s, d_in,
+                      static_cast<typename Elem<S>::T *>(f), cells, h->args);
   });
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "set populations");
@@ -1976,15 +2034,16 @@ extern "C" int lesbgk_moments_rows(lesbgk *h, int32_t j0, int32_t nrows, float *
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const void *f = h->buf[h->cur];
   const long long cells = (long long)nrows * h->p.nx;
+  const unsigned blocks = mom_blocks(cells);
   dispatch(h->nr, h->order, h->p.storage, h->p.dim, [&](auto r, auto, auto st, auto z) {
     constexpr int NR = decltype(r)::value, NZ = decltype(z)::value;
     using S = decltype(st);
     using E = typename Elem<S>::T;
     constexpr int V = Layout<NR, E, NZ>::V;  // (for Comp the hi plane's; the lo plane shares its byte offsets)
     const E *fr = static_cast<const E *>(f) + (long long)j0 * h->p.nx * V;
-    k_moments<NR, S, NZ><<<kMomGrid, kMomBlock, 0, s>>>(fr, d_out, h->partial, cells, h->args.plane, h->args);
+    launch_overlapped(k_moments<NR, S, NZ>, blocks, kMomBlock, s, fr, d_out, h->partial, cells, h->args.plane, h->args);
   });
-  k_reduce_partials<<<1, 128, 0, s>>>(h->partial, kMomGrid, h->sums);
+  if (h_sums) launch_overlapped(k_reduce_partials, 1, 128, s, h->partial, (int)blocks, h->sums);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "moments of rows");
   return finish_sums(h, h_sums, s);
