@@ -1338,26 +1338,26 @@ int pick_launch(lesbgk *h) {
   // One node per lane, 28 nodes per strip (two halo lanes per side).  Rows per
   // segment: a segment costs its rows plus a prologue (the stencil rows and
   // the ring's first loads, about kPro rows' time); a row takes one warp's
-  // latency or, with k blocks on the SM, k times a block's `share` of the
-  // issue slots, whichever is more (one-block against full-chip runs, in units
-  // of that latency); past one wave the blocks' ends are spread over half a
-  // segment.  Small grids so get short segments, middle ones the longest that
+  // latency or, with k blocks on the SM, `base` + k times a block's `share` of
+  // the issue slots, whichever is more (one-block against full-chip runs, in
+  // units of that latency); past one wave the blocks' ends are spread over half
+  // a segment.  Small grids so get short segments, middle ones the longest that
   // fill every SM evenly (us per step with 32 or, D2Q36 and D3Q216, 128 rows ->
   // now; 4x64 D2Q16 18.6 -> 2.7, D2Q36 70 -> 4.2; 256^2 cavity 25.6 -> 4.9;
-  // 512x1024 D2Q16 19.8 -> 14.8; 512^2 D2Q36 140 -> 18.0, D3Q64 33.0 -> 15.5).
+  // 512x1024 D2Q16 19.8 -> 14.3; 512^2 D2Q36 140 -> 18.0, D3Q64 33.0 -> 15.5).
   // From two waves of `large` rows on, `large` is taken: 16 to 128 rows are
   // within 4% there (4096^2 D2Q16: 367, 354, 361, 365 us at 16, 32, 64, 128;
   // D3Q64: 808, 775, 777, 770).
   constexpr double kPro = 1.5;
   const bool comp = h->p.storage == LESBGK_F32C, wide = h->q >= 32;
   const double slots = wide ? 2 : comp ? 3 : 4;  // blocks an SM holds (registers)
-  const double share = wide ? 0.85 : comp ? 0.70 : 0.63;
+  const double share = wide ? 0.85 : comp ? 0.70 : 0.46, base = wide || comp ? 0.0 : 0.42;
   const int large = wide && !comp ? 128 : 32;
   h->cpt = 1;
   const int nstrips = (nx + 27) / 28;
   if (h->rows <= 0) {
     const double sms = h->sm_count > 0 ? h->sm_count : 152;
-    const double cap = slots * sms, full = share * slots;
+    const double cap = slots * sms, full = base + share * slots;
     const double per_block = h->q >= 100 ? 1 : kBlock / 32;  // strips (D3Q216: one)
     h->rows = large < ny ? large : ny;
     if ((double)nstrips * ny < 2.0 * large * cap * per_block) {
@@ -1372,7 +1372,7 @@ int pick_launch(lesbgk *h) {
         // SM gets a full set (1024^2 compensated: two of three slots, 32 rows,
         // 56 us per step; three of three, 21 rows, 40 us)
         if (2.0 * k > slots) k = slots;
-        if (blocks <= cap) t = (r + kPro) * std::fmax(1.0, share * k);
+        if (blocks <= cap) t = (r + kPro) * std::fmax(1.0, base + share * k);
         else if (whole <= cap) t = (r + kPro) * full + rest + kPro;  // the short segments follow the full wave
         else t = full * (r + kPro) * (blocks / cap + 0.5);
         if (r == 1 || t <= best) {
