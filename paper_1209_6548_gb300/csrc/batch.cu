@@ -332,9 +332,10 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
       S *o = fout + (long long)j * rstride + (long long)lx * V;
       if constexpr (Store<S>::kScaled) {  // the key of k_step: step count and row
         const unsigned seed = (unsigned)B.nstep[2 * fl.w + par] * 0x9e3779b9u + 0x7f4a7c15u;
-        const unsigned key = mix32(seed ^ mix32((unsigned)j));
+        const unsigned key = round_key(seed, j);
 #pragma unroll
-        for (int g = 0; g < G; ++g) st_group_sr<NR, S>(o, gstride, g, acc, B.lat, key);
+        for (int g = 0; g < G; ++g)
+          *reinterpret_cast<T *>(o + g * gstride) = pack_group_sr<NR, S>(g, acc, B.lat, group_word(key, g));
       } else {
 #pragma unroll
         for (int g = 0; g < G; ++g) st_group_s<NR, S>(o, gstride, g, acc, B.lat);

@@ -834,33 +834,32 @@ __device__ __forceinline__ void st_group_s(S *p, long long gstride, int g, const
   *reinterpret_cast<R *>(p + g * gstride) = raw;
 }
 
-// Store with stochastic rounding for the 16-bit types (FP32 stores as is):
-// pairs of values go through the hardware's stochastic rounding (cvt.rs,
-// unbiased for both halves), fed one 32-bit random word per pair: the first
-// is mix32(key ^ g * 0x9e3779b9), each next one a multiply-add of the last
-// (each word is a bijection of a uniform seed, hence uniform).  Results depend
-// only on the key and the population, never on the launch shape.
+// Stored form of a group with stochastic rounding for the 16-bit types: pairs
+// of values go through the hardware's stochastic rounding (cvt.rs, unbiased
+// for both halves), fed one 32-bit random word per pair: the group's word
+// first, each next one a multiply-add of the last (each word is a bijection of
+// a uniform seed, hence uniform).  Results depend only on the words and the
+// population, never on the launch shape.
 template <int NR, class S, int Q, class TT>
-__device__ __forceinline__ void st_group_sr(S *p, long long gstride, int g, const float (&F)[Q],
-                                            const TT &Tt, unsigned key) {
-  if constexpr (!Store<S>::kScaled) {
-    st_group_s<NR, S>(p, gstride, g, F, Tt);
-  } else {
-    using L = LayoutQ<NR, S, Q>;
-    static_assert(L::V % 2 == 0, "16-bit groups hold pairs");
-    using R = typename Raw<L::VB>::T;
-    R raw;
-    unsigned *w = reinterpret_cast<unsigned *>(&raw);
-    unsigned bits = mix32(key ^ ((unsigned)g * 0x9e3779b9u));
+__device__ __forceinline__ typename Raw<LayoutQ<NR, S, Q>::VB>::T pack_group_sr(int g, const float (&F)[Q], const TT &Tt,
+                                                                                unsigned bits) {
+  using L = LayoutQ<NR, S, Q>;
+  static_assert(L::V % 2 == 0, "16-bit groups hold pairs");
+  typename Raw<L::VB>::T raw;
+  unsigned *w = reinterpret_cast<unsigned *>(&raw);
 #pragma unroll
-    for (int k = 0; k < L::V; k += 2) {
-      const int a0 = L::alpha(g * L::V + k), a1 = L::alpha(g * L::V + k + 1);
-      w[k / 2] = Store<S>::put_sr2(F[a0] * Tt.iwq[a0], F[a1] * Tt.iwq[a1], bits);
-      bits = bits * 0x9e3779b5u + 0x7f4a7c15u;
-    }
-    *reinterpret_cast<R *>(p + g * gstride) = raw;
+  for (int k = 0; k < L::V; k += 2) {
+    const int a0 = L::alpha(g * L::V + k), a1 = L::alpha(g * L::V + k + 1);
+    w[k / 2] = Store<S>::put_sr2(F[a0] * Tt.iwq[a0], F[a1] * Tt.iwq[a1], bits);
+    bits = bits * 0x9e3779b5u + 0x7f4a7c15u;
   }
+  return raw;
 }
+
+// The random word of a row's group g: the row's key (of the step and the row)
+// mixed with the group.
+__device__ __forceinline__ unsigned round_key(unsigned seed, int row) { return mix32(seed ^ mix32((unsigned)row)); }
+__device__ __forceinline__ unsigned group_word(unsigned key, int g) { return mix32(key ^ ((unsigned)g * 0x9e3779b9u)); }
 
 // ---------------------------------------------------------------------------
 // Compensated FP32 storage (tag Comp): each stored deviation is hi + lo, hi an

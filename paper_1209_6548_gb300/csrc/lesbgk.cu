@@ -47,6 +47,18 @@ constexpr int kMomBlock = 256;
 // ---------------------------------------------------------------------------
 // The fused time step (Sec. 3.1 + Sec. 3.2).
 // ---------------------------------------------------------------------------
+// Rounding key per step and row (not per column): a flow uniform in x stays
+// exactly uniform, so rounding noise cannot seed the x-varying modes the
+// printed unsplit update amplifies.
+__device__ __forceinline__ unsigned row_rounding_key(const KArgs &A, int row) {
+  int gr = row + A.row_key;  // the global row (a y-slab's halo rows may wrap around)
+  if (A.row_period) {
+    gr %= A.row_period;
+    if (gr < 0) gr += A.row_period;
+  }
+  return round_key(A.seed, gr);
+}
+
 template <int NR, int N, bool SPLIT, int RING, class S, int WM, int NZ = 1>
 __global__ void __launch_bounds__(kBlock) k_step(const S *__restrict__ fin, S *__restrict__ fout,
                                                  const KArgs A) {
@@ -130,8 +142,21 @@ __global__ void __launch_bounds__(kBlock) k_step(const S *__restrict__ fin, S *_
 #pragma unroll
   for (int k = 0; k < RING - 1; ++k) issue_rowload(k);
 
+  // The random words of 16-bit rounding depend on the row alone.  With two
+  // groups per node (D2Q16) a warp computes them for 32 rows at a time, a row
+  // per lane, and reads them back with a shuffle, outside the writers' branch
+  // (4096^2: FP16 407.5 -> 399.4 us, BF16 410.3 -> 403.9); with more groups the
+  // shuffles cost as much (D3Q64 221.6 -> 224.0 at 2048^2, D2Q36 290.8 -> 325).
+  constexpr bool kRowWords = Store<S>::kScaled && G <= 2;
+  [[maybe_unused]] unsigned words[kRowWords ? G : 1];
   for (int j = y0; j < y1; ++j) {
     const int k = j - y0;
+    if constexpr (kRowWords)
+      if (k % 32 == 0) {
+        const unsigned key = row_rounding_key(A, j + lane);
+#pragma unroll
+        for (int g = 0; g < G; ++g) words[g] = group_word(key, g);
+      }
     issue_rowload(k + RING - 1);
     cp_async_wait<RING - 1>();  // row-load k has landed
     float ld[Q];
@@ -196,19 +221,24 @@ __global__ void __launch_bounds__(kBlock) k_step(const S *__restrict__ fin, S *_
     // instantiations so that the hot loop of everything else keeps its code
     apply_walls_node<NR, WM>(acc, xw, j, A);
 
-    if (writer) {
-      S *o = fout + (long long)j * rstride + (long long)xw * V;
-      // rounding key per step and row (not per column): a flow uniform in x stays
-      // exactly uniform, so rounding noise cannot seed the x-varying modes the
-      // printed unsplit update amplifies
-      int gr = j + A.row_key;  // the global row (a y-slab's halo rows may wrap around)
-      if (A.row_period) {
-        gr %= A.row_period;
-        if (gr < 0) gr += A.row_period;
-      }
-      const unsigned key = mix32(A.seed ^ mix32((unsigned)gr));
+    S *o = fout + (long long)j * rstride + (long long)xw * V;
+    if constexpr (kRowWords) {
 #pragma unroll
-      for (int g = 0; g < G; ++g) st_group_sr<NR, S>(o, gstride, g, acc, A, key);
+      for (int g = 0; g < G; ++g) {
+        const unsigned bits = __shfl_sync(kFull, words[g], k & 31);
+        const auto raw = pack_group_sr<NR, S>(g, acc, A, bits);
+        if (writer) *reinterpret_cast<T *>(o + g * gstride) = raw;
+      }
+    } else if (writer) {
+      if constexpr (Store<S>::kScaled) {
+        const unsigned key = row_rounding_key(A, j);
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+          *reinterpret_cast<T *>(o + g * gstride) = pack_group_sr<NR, S>(g, acc, A, group_word(key, g));
+      } else {
+#pragma unroll
+        for (int g = 0; g < G; ++g) st_group_s<NR, S>(o, gstride, g, acc, A);
+      }
     }
   }
   cp_async_wait<0>();
@@ -524,19 +554,14 @@ __global__ void __launch_bounds__(kBlockZ) k_step_z(const S *__restrict__ fin, S
     if (writer) {
       S *o = fout + (long long)j * rstride + (long long)xw * V;
       if constexpr (kScaled) {
-        // the random words of st_group_sr: one per pair, keyed by the step,
-        // the global row and the node's group (9 iz + g, or 18 + 9 iz + g)
-        int gr = j + A.row_key;
-        if (A.row_period) {
-          gr %= A.row_period;
-          if (gr < 0) gr += A.row_period;
-        }
-        const unsigned key = mix32(A.seed ^ mix32((unsigned)gr));
+        // the random words of the one-thread layout: one per pair, keyed by the
+        // step, the global row and the node's group (9 iz + g, or 18 + 9 iz + g)
+        const unsigned key = row_rounding_key(A, j);
 #pragma unroll
         for (int g = 0; g < GL; ++g) {
           const int a0 = LL::alpha(g * V), a1 = LL::alpha(g * V + 1);
           const int gg = 9 * iz + g + (g < GL / 2 ? 0 : 18);
-          const unsigned bits = mix32(key ^ ((unsigned)gg * 0x9e3779b9u));
+          const unsigned bits = group_word(key, gg);
           *reinterpret_cast<T *>(o + (g < GL / 2 ? lo : hi) + g * gstride) =
               Store<S>::put_sr2(acc[a0] * A.iwq[zo + a0], acc[a1] * A.iwq[zo + a1], bits);
         }
