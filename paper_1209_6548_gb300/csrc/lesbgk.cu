@@ -59,7 +59,9 @@ __device__ __forceinline__ unsigned row_rounding_key(const KArgs &A, int row) {
   return round_key(A.seed, gr);
 }
 
-template <int NR, int N, bool SPLIT, int RING, class S, int WM, int NZ = 1>
+// EARLY: the ring's first loads go out before the stencil rows are read, so
+// that a segment waits for memory once, not twice.
+template <int NR, int N, bool SPLIT, int RING, class S, int WM, int NZ, bool EARLY>
 __global__ void __launch_bounds__(kBlock) k_step(const S *__restrict__ fin, S *__restrict__ fout,
                                                  const KArgs A) {
   using Lay = Layout<NR, S, NZ>;
@@ -90,15 +92,54 @@ __global__ void __launch_bounds__(kBlock) k_step(const S *__restrict__ fin, S *_
   // rows), never per population.
   auto row_ptr = [&](int j) { return fx + map_row(j, ny, A.walls) * rstride; };
 
+  // Look-ahead rows go through a per-lane ring of RING row slots in shared
+  // memory, filled by asynchronous copies (cp.async, one vector per group):
+  // RING-1 rows are in flight while a row is processed, without holding
+  // registers.  Each lane copies and reads only its own node's vectors, so the
+  // ring needs no barrier; cp.async.wait_group paces it.  "Row-load k" holds
+  // what row y0+k consumes: f_{j+1} for c_y > 0 groups, f_{j+2} for c_y < 0.
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  using T = typename Raw<Lay::VB>::T;
+  T *ring = reinterpret_cast<T *>(smem_raw) + (size_t)(threadIdx.x >> 5) * RING * G * 32 + lane;
+  int r1, r2;
+  const int nrows = y1 - y0;
+  auto issue_rowload = [&](int k) {
+    if (k < nrows) {
+      const S *q1 = fx + r1 * rstride, *q2 = fx + r2 * rstride;
+      T *slot = ring + (k % RING) * G * 32;
+#pragma unroll
+      for (int g = 0; g < G; ++g) cp_async_raw<Lay::VB>(slot + g * 32, (g >= G / 2 ? q1 : q2) + g * gstride);
+      r1 = r2;
+      r2 = r2 + 1 < ny ? r2 + 1 : (A.walls ? ny - 1 : 0);
+    }
+    cp_async_commit();  // (an empty group past the segment end keeps the count uniform)
+  };
+  int row0[4] = {y0 - 2, y0 - 1, y0, y0 + 1};
+  if constexpr (EARLY) {  // the rows are resolved while the previous step still runs
+    r1 = map_row(y0 + 1, ny, A.walls);
+    r2 = map_row(y0 + 2, ny, A.walls);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      row0[i] = map_row(row0[i], ny, A.walls);
+      asm volatile("" : "+r"(row0[i]));
+    }
+    asm volatile("" : "+r"(r1), "+r"(r2));
+  }
+  pdl_wait();
+  pdl_trigger();
+  if constexpr (EARLY) {
+#pragma unroll
+    for (int k = 0; k < RING - 1; ++k) issue_rowload(k);
+  }
+
   // y-stencil state per population:
   //   c_y > 0: s0 = f_j - f_{j-1}, s1 = sigma_{j-1}; fc = f_j
   //   c_y < 0: s0 = f_{j+1},       s1 = sigma_j;     fc = f_j
-  pdl_wait();
-  pdl_trigger();
   float fc[Q], s0[Q], s1[Q];
   {
     float m2[Q], m1[Q], p1[Q];
-    const S *pm2 = row_ptr(y0 - 2), *pm1 = row_ptr(y0 - 1), *pz = row_ptr(y0), *pp1 = row_ptr(y0 + 1);
+    auto stencil_row = [&](int i) { return EARLY ? fx + row0[i] * rstride : row_ptr(row0[i]); };
+    const S *pm2 = stencil_row(0), *pm1 = stencil_row(1), *pz = stencil_row(2), *pp1 = stencil_row(3);
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       ld_group_cg<NR, S>(pm1, gstride, g, m1, A);
@@ -117,30 +158,12 @@ __global__ void __launch_bounds__(kBlock) k_step(const S *__restrict__ fin, S *_
       }
     }
   }
-  // Look-ahead rows go through a per-lane ring of RING row slots in shared
-  // memory, filled by asynchronous copies (cp.async, one vector per group):
-  // RING-1 rows are in flight while a row is processed, without holding
-  // registers.  Each lane copies and reads only its own node's vectors, so the
-  // ring needs no barrier; cp.async.wait_group paces it.  "Row-load k" holds
-  // what row y0+k consumes: f_{j+1} for c_y > 0 groups, f_{j+2} for c_y < 0.
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  using T = typename Raw<Lay::VB>::T;
-  T *ring = reinterpret_cast<T *>(smem_raw) + (size_t)(threadIdx.x >> 5) * RING * G * 32 + lane;
-  int r1 = map_row(y0 + 1, ny, A.walls), r2 = map_row(y0 + 2, ny, A.walls);
-  const int nrows = y1 - y0;
-  auto issue_rowload = [&](int k) {
-    if (k < nrows) {
-      const S *q1 = fx + r1 * rstride, *q2 = fx + r2 * rstride;
-      T *slot = ring + (k % RING) * G * 32;
+  if constexpr (!EARLY) {
+    r1 = map_row(y0 + 1, ny, A.walls);
+    r2 = map_row(y0 + 2, ny, A.walls);
 #pragma unroll
-      for (int g = 0; g < G; ++g) cp_async_raw<Lay::VB>(slot + g * 32, (g >= G / 2 ? q1 : q2) + g * gstride);
-      r1 = r2;
-      r2 = r2 + 1 < ny ? r2 + 1 : (A.walls ? ny - 1 : 0);
-    }
-    cp_async_commit();  // (an empty group past the segment end keeps the count uniform)
-  };
-#pragma unroll
-  for (int k = 0; k < RING - 1; ++k) issue_rowload(k);
+    for (int k = 0; k < RING - 1; ++k) issue_rowload(k);
+  }
 
   // The random words of 16-bit rounding depend on the row alone.  With two
   // groups per node (D2Q16) a warp computes them for 32 rows at a time, a row
@@ -309,7 +332,6 @@ __global__ void __launch_bounds__(kBlockZ) k_step_z(const S *__restrict__ fin, S
   // groups at 27 + 9 iz + (gl - 9)
   const long long lo = (long long)(9 * iz) * gstride, hi = (long long)(18 + 9 * iz) * gstride;
   const S *fx = fin + (long long)xw * V;
-  auto row_ptr = [&](int j) { return fx + map_row(j, ny, A.walls) * rstride; };
   // a level's raw vector -> FP32 deviations (scale of stored population zo + a)
   auto unpack_z = [&](const T &raw, int g, float (&F)[Q]) {
     const S *e = reinterpret_cast<const S *>(&raw);
@@ -324,12 +346,22 @@ __global__ void __launch_bounds__(kBlockZ) k_step_z(const S *__restrict__ fin, S
     unpack_z(raw, g, F);
   };
 
+  // the rows are resolved while the previous step still runs
+  int row0[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    row0[i] = map_row(y0 - 2 + i, ny, A.walls);
+    asm volatile("" : "+r"(row0[i]));
+  }
+  int r1 = map_row(y0 + 1, ny, A.walls), r2 = map_row(y0 + 2, ny, A.walls);
+  asm volatile("" : "+r"(r1), "+r"(r2));
   pdl_wait();
   pdl_trigger();
   float fc[Q], s0[Q], s1[Q];
   {
     float m2[Q], m1[Q], p1[Q];
-    const S *pm2 = row_ptr(y0 - 2), *pm1 = row_ptr(y0 - 1), *pz = row_ptr(y0), *pp1 = row_ptr(y0 + 1);
+    const S *pm2 = fx + row0[0] * rstride, *pm1 = fx + row0[1] * rstride, *pz = fx + row0[2] * rstride,
+            *pp1 = fx + row0[3] * rstride;
 #pragma unroll
     for (int g = 0; g < GL; ++g) {
       const long long off = g < GL / 2 ? lo : hi;
@@ -358,7 +390,6 @@ __global__ void __launch_bounds__(kBlockZ) k_step_z(const S *__restrict__ fin, S
   // this level's z-weights, read once: 2 He_2(c_z) and w_z He_l(c_z)/l!, l = 0, 2, 4
   const float he2 = 2.0f * A.he[H + iz][2];
   const float hz[3] = {A.hw[H + iz][0], A.hw[H + iz][2], A.hw[H + iz][4]};
-  int r1 = map_row(y0 + 1, ny, A.walls), r2 = map_row(y0 + 2, ny, A.walls);
   const int nrows = y1 - y0;
   auto issue_rowload = [&](int k) {
     if (k < nrows) {
@@ -640,7 +671,7 @@ __global__ void __launch_bounds__(kBlock, NZ == 1 ? 3 : 1) k_step_c(const float 
     }
   };
   auto load_row = [&](int j, float (&hi)[Q], float (&lo)[Q]) {
-    const uint4 *p = vx + (long long)map_row(j, ny, A.walls) * nx;
+    const uint4 *p = vx + (long long)j * nx;
     uint4 v[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) v[g] = __ldcg(p + g * plane);
@@ -650,15 +681,24 @@ __global__ void __launch_bounds__(kBlock, NZ == 1 ? 3 : 1) k_step_c(const float 
   // y-stencil per population, as in k_step, with hi and lo parts of values:
   //   c_y > 0: s0 = f_j - f_{j-1} (a difference), s1 = sigma_{j-1}; fc = f_j
   //   c_y < 0: s0 = f_{j+1} (s0h + s0l),        s1 = sigma_j;     fc = f_j
+  // the rows are resolved while the previous step still runs
+  int row0[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    row0[i] = map_row(y0 - 2 + i, ny, A.walls);
+    asm volatile("" : "+r"(row0[i]));
+  }
+  int r1 = map_row(y0 + 1, ny, A.walls), r2 = map_row(y0 + 2, ny, A.walls);
+  asm volatile("" : "+r"(r1), "+r"(r2));
   pdl_wait();
   pdl_trigger();
   float fch[Q], fcl[Q], s0h[Q], s0l[Q], s1[Q];
   {
     float m2h[Q], m2l[Q], m1h[Q], m1l[Q], p1h[Q], p1l[Q];
-    load_row(y0 - 2, m2h, m2l);
-    load_row(y0 - 1, m1h, m1l);
-    load_row(y0, fch, fcl);
-    load_row(y0 + 1, p1h, p1l);
+    load_row(row0[0], m2h, m2l);
+    load_row(row0[1], m1h, m1l);
+    load_row(row0[2], fch, fcl);
+    load_row(row0[3], p1h, p1l);
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
       const float d0 = (fch[a] - m1h[a]) + (fcl[a] - m1l[a]);  // f_j - f_{j-1}
@@ -675,7 +715,6 @@ __global__ void __launch_bounds__(kBlock, NZ == 1 ? 3 : 1) k_step_c(const float 
   }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint4 *ring = reinterpret_cast<uint4 *>(smem_raw) + (size_t)(threadIdx.x >> 5) * RING * G * 32 + lane;
-  int r1 = map_row(y0 + 1, ny, A.walls), r2 = map_row(y0 + 2, ny, A.walls);
   const int nrows = y1 - y0;
   auto issue_rowload = [&](int k) {
     if (k < nrows) {
@@ -1153,14 +1192,6 @@ __global__ void __launch_bounds__(NR == 4 && NZ == 1 ? 512 : 256, 1)
   const int slots = (most + 4) * nx;        // nodes of a group plane: row slot s holds row a0 - 2 + s
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *buf = reinterpret_cast<T *>(smem_raw);  // [2][G][slots]
-  pdl_wait();
-  pdl_trigger();
-  for (int t = threadIdx.x; t < (b0 - a0 + 4) * nx; t += blockDim.x) {
-    const int j = map_row(a0 - 2 + t / nx, ny, A.walls);
-    const T *p = reinterpret_cast<const T *>(f) + (long long)j * nx + t % nx;
-#pragma unroll
-    for (int g = 0; g < G; ++g) buf[g * slots + t] = __ldcg(p + g * A.plane);
-  }
   const int lane = threadIdx.x & 31;
   const int per = 32 / nx;                       // rows a warp takes
   const int gi = min(lane / nx, per - 1), x = lane % nx;
@@ -1192,6 +1223,14 @@ __global__ void __launch_bounds__(NR == 4 && NZ == 1 ? 512 : 256, 1)
     } else if (!whigh && b0 - j <= 2) {
       extra[1] = at(rank + 1 < ctas ? rank + 1 : 0, 2 - (b0 - j));
     }
+  }
+  pdl_wait();
+  pdl_trigger();
+  for (int t = threadIdx.x; t < (b0 - a0 + 4) * nx; t += blockDim.x) {
+    const int j = map_row(a0 - 2 + t / nx, ny, A.walls);
+    const T *p = reinterpret_cast<const T *>(f) + (long long)j * nx + t % nx;
+#pragma unroll
+    for (int g = 0; g < G; ++g) buf[g * slots + t] = __ldcg(p + g * A.plane);
   }
   auto sync = [&] {
     if (ctas > 1) cluster_barrier();
@@ -1430,6 +1469,16 @@ int build_tables(lesbgk *h, const FieldStats *stats) {
 
 constexpr int kRing = 4;
 
+// The order of k_step's first loads.  EARLY (rows resolved before the wait for
+// the previous step, ring loads before the stencil rows) is the faster one on
+// short segments (us per step, late -> early: 64^2 2.81 -> 2.18, 512^2 8.58 ->
+// 8.09, 512x1024 14.27 -> 14.05, 512^2 D2Q36 18.0 -> 17.6) and for D2Q36 and
+// FP32 D3Q64 on all (1999x2053 D3Q64 197.7 -> 195.7); from 24 rows on the late
+// order is ahead on the sets that have both (4096^2 FP32 354.5 against 355.4,
+// FP16 398.3 against 400.3).
+template <int NR, class S, int NZ>
+constexpr bool kLateToo = NR == 4 && (NZ == 1 || !std::is_same<S, float>::value);
+
 template <int NR, class S, int NZ>
 constexpr size_t step_smem_bytes() {
   if constexpr (kIsComp<S>)  // both planes' 16-byte vectors
@@ -1500,14 +1549,19 @@ cudaError_t allow_smem(const lesbgk *h) {
       allow(k_step_z<false, kRing, 2, S>, smem);
     } else {
       constexpr int smem = (int)step_smem_bytes<NR, S, NZ>();
-      allow(k_step<NR, N, true, kRing, S, 0, NZ>, smem);
-      allow(k_step<NR, N, false, kRing, S, 0, NZ>, smem);
-      allow(k_step<NR, N, true, kRing, S, 2, NZ>, smem);
-      allow(k_step<NR, N, false, kRing, S, 2, NZ>, smem);
-      if constexpr (std::is_same<S, float>::value) {
-        allow(k_step<NR, N, true, kRing, S, 1, NZ>, smem);
-        allow(k_step<NR, N, false, kRing, S, 1, NZ>, smem);
-      }
+      auto allow_both = [&](auto early) {
+        constexpr bool E = decltype(early)::value;
+        allow(k_step<NR, N, true, kRing, S, 0, NZ, E>, smem);
+        allow(k_step<NR, N, false, kRing, S, 0, NZ, E>, smem);
+        allow(k_step<NR, N, true, kRing, S, 2, NZ, E>, smem);
+        allow(k_step<NR, N, false, kRing, S, 2, NZ, E>, smem);
+        if constexpr (std::is_same<S, float>::value) {
+          allow(k_step<NR, N, true, kRing, S, 1, NZ, E>, smem);
+          allow(k_step<NR, N, false, kRing, S, 1, NZ, E>, smem);
+        }
+      };
+      allow_both(std::true_type{});
+      if constexpr (kLateToo<NR, S, NZ>) allow_both(std::false_type{});
     }
   });
   return e;
@@ -1565,20 +1619,29 @@ int launch_step(lesbgk *h, const void *fin, void *fout, bool overlap, cudaStream
       return;
     } else {
       constexpr size_t smem = step_smem_bytes<NR, S, NZ>();
-      if (h->args.xwalls) {  // walls in x (cavity)
-        if (split) go(k_step<NR, N, true, kRing, S, 2, NZ>, grid, kBlock, smem);
-        else go(k_step<NR, N, false, kRing, S, 2, NZ>, grid, kBlock, smem);
-        return;
-      }
-      if constexpr (std::is_same<S, float>::value) {  // Maxwell walls: FP32 storage (checked at set-up)
-        if (h->args.walls && h->args.wspec != 0.0f) {  // Maxwell walls
-          if (split) go(k_step<NR, N, true, kRing, S, 1, NZ>, grid, kBlock, smem);
-          else go(k_step<NR, N, false, kRing, S, 1, NZ>, grid, kBlock, smem);
+      auto run = [&](auto early) {
+        constexpr bool E = decltype(early)::value;
+        if (h->args.xwalls) {  // walls in x (cavity)
+          if (split) go(k_step<NR, N, true, kRing, S, 2, NZ, E>, grid, kBlock, smem);
+          else go(k_step<NR, N, false, kRing, S, 2, NZ, E>, grid, kBlock, smem);
           return;
         }
+        if constexpr (std::is_same<S, float>::value) {  // Maxwell walls: FP32 storage (checked at set-up)
+          if (h->args.walls && h->args.wspec != 0.0f) {
+            if (split) go(k_step<NR, N, true, kRing, S, 1, NZ, E>, grid, kBlock, smem);
+            else go(k_step<NR, N, false, kRing, S, 1, NZ, E>, grid, kBlock, smem);
+            return;
+          }
+        }
+        if (split) go(k_step<NR, N, true, kRing, S, 0, NZ, E>, grid, kBlock, smem);
+        else go(k_step<NR, N, false, kRing, S, 0, NZ, E>, grid, kBlock, smem);
+      };
+      if constexpr (kLateToo<NR, S, NZ>) {
+        if (h->rows >= 24) run(std::false_type{});
+        else run(std::true_type{});
+      } else {
+        run(std::true_type{});
       }
-      if (split) go(k_step<NR, N, true, kRing, S, 0, NZ>, grid, kBlock, smem);
-      else go(k_step<NR, N, false, kRing, S, 0, NZ>, grid, kBlock, smem);
     }
   });
   return 0;
