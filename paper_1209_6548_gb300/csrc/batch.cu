@@ -1,6 +1,7 @@
 // Batched lattice ES-BGK solver: many independent narrow solves (nx a power of
 // two <= 32, e.g. the 1D-in-y channel flows of Sec. 4 of the paper) advanced
-// together, one launch per lattice per time step, replayed from CUDA graphs.
+// together, one launch per class and chain per time step, replayed from CUDA
+// graphs.
 //
 // Device memory: the caller's workspace holds fixed tables (per-slot
 // descriptors, the work list, residual and moment scratch) and a pool from
@@ -743,7 +744,7 @@ struct lesbgk_batch {
   InstDesc *d_desc = nullptr;
   WorkItem *d_items = nullptr;
   int *d_range = nullptr;      // {first, count} per class of the items the per-step kernel takes, then per class and chain
-  int *d_range_all = nullptr;  // {first, count} per class of all items (residuals, moments)
+  int *d_range_all = nullptr;  // {first, count} per class of the items that cover every solve (residuals, moments)
   int *d_rlist = nullptr;      // resident instances, bucket after bucket
   int *d_rrange = nullptr;     // {first, count} per bucket
   unsigned *d_res = nullptr;
@@ -756,7 +757,8 @@ struct lesbgk_batch {
   size_t pool_bytes = 0;
   Pool pool;
   std::vector<Slot> slots;
-  std::vector<WorkItem> items;
+  std::vector<WorkItem> items;  // on the device in this order
+  size_t read_items = 0;        // the first so many are what residuals and moments go over
   int range[kNumClasses][2] = {};
   int range_all[kNumClasses][2] = {};
   int rrange[kBuckets][2] = {};
@@ -886,8 +888,8 @@ BatchArgs make_args(const lesbgk_batch *b, int cls) {
   return a;
 }
 
-// The same over every item of the class, resident instances included
-// (residuals, moments).
+// The same over the items that cover every solve of the class (residuals,
+// moments).
 BatchArgs make_args_all(const lesbgk_batch *b, int cls) {
   BatchArgs a = make_args(b, cls);
   a.range = b->d_range_all + 2 * cls;
@@ -999,9 +1001,9 @@ void pick_rows(lesbgk_batch *b) {
 }
 
 // Rebuild the host work list and copy it with the class ranges to the device:
-// per class, the items of the instances the per-step kernel takes (sorted by
-// length), then those of the resident instances (whose items only the
-// residual and moment kernels visit); and the resident instances by bucket.
+// the items that residuals and moments go over, then per class and chain those
+// of the instances the per-step kernel takes (sorted by length); and the
+// resident instances by bucket.
 int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
   b->items.clear();
   if (b->auto_resident) {
@@ -1010,6 +1012,23 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
       if (sl.used && (sl.cls != 0 || sl.p.ny > std::min(b->resident_ny, kAutoResidentNy))) b->resident = false;
   }
   pick_rows(b);
+  // Residuals and moments read every solve in items of their own, of the
+  // default rows (one node per thread), where the steps' rows are the rule's;
+  // otherwise both go over one list.  Each list has half of a solve's room.
+  const bool own = b->auto_rows;
+  const size_t room = own ? kItemsPerSlot / 2 : kItemsPerSlot;
+  auto rows_in_room = [&](int rows, int ny) { return std::max(rows, (int)((ny + room - 1) / room)); };
+  for (int cls = 0; own && cls < kNumClasses; ++cls) {
+    b->range_all[cls][0] = (int)b->items.size();
+    for (int i = 0; i < b->capacity; ++i) {
+      const auto &sl = b->slots[i];
+      if (!sl.used || sl.cls != cls) continue;
+      const int r = rows_in_room(b->rows, sl.p.ny);
+      for (int y0 = 0; y0 < sl.p.ny; y0 += r) b->items.push_back({i, y0, std::min(r, sl.p.ny - y0), 0});
+    }
+    b->range_all[cls][1] = (int)b->items.size() - b->range_all[cls][0];
+  }
+  b->read_items = b->items.size();
   for (int cls = 0; cls < kNumClasses; ++cls) {
     const int first = (int)b->items.size();
     std::vector<WorkItem> mine[kChains], res;
@@ -1021,10 +1040,10 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
     long long load[kChains] = {};
     for (int i : order) {
       const auto &sl = b->slots[i];
-      // (a tall solve keeps within its room of the work list)
-      const int r = std::max(b->rows_of[cls], (int)((sl.p.ny + kItemsPerSlot - 1) / kItemsPerSlot));
+      const int r = rows_in_room(b->rows_of[cls], sl.p.ny);
       const int c = (int)(std::min_element(load, load + b->chains_of[cls]) - load);
       if (!is_resident(b, sl)) load[c] += sl.p.ny;
+      if (own && is_resident(b, sl)) continue;
       auto &dst = is_resident(b, sl) ? res : mine[c];
       for (int y0 = 0; y0 < sl.p.ny; y0 += r) dst.push_back({i, y0, std::min(r, sl.p.ny - y0), 0});
     }
@@ -1038,9 +1057,12 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
     b->items.insert(b->items.end(), res.begin(), res.end());
     b->range[cls][0] = first;
     b->range[cls][1] = stepped;
-    b->range_all[cls][0] = first;
-    b->range_all[cls][1] = stepped + (int)res.size();
+    if (!own) {
+      b->range_all[cls][0] = first;
+      b->range_all[cls][1] = stepped + (int)res.size();
+    }
   }
+  if (!own) b->read_items = b->items.size();
   if ((long long)b->items.size() > (long long)b->capacity * (long long)kItemsPerSlot)
     return fail(LESBGK_ESPACE, "work list of %zu items exceeds its room", b->items.size());
   std::vector<int> rlist;
@@ -1404,8 +1426,8 @@ extern "C" int lesbgk_batch_add_many(lesbgk_batch *b, int32_t n, const lesbgk_pa
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
   if (!rc && n) {
-    // the descriptors of the touched range in one copy, the fields one by one,
-    // then one init launch per lattice class over the new slots
+    // the descriptors of the touched range in one copy, then fields and init
+    // launches below
     const int lo = *std::min_element(taken.begin(), taken.end());
     const int hi = *std::max_element(taken.begin(), taken.end());
     std::vector<InstDesc> desc(hi - lo + 1);
@@ -1550,7 +1572,7 @@ extern "C" int lesbgk_batch_residuals(lesbgk_batch *b, double *h_res, double *h_
     e = cudaGetLastError();
   }
   std::vector<unsigned> bits(b->capacity);
-  std::vector<double> part(h_mass ? b->items.size() : 0);
+  std::vector<double> part(h_mass ? b->read_items : 0);
   if (e == cudaSuccess) e = cudaMemcpyAsync(bits.data(), b->d_res, sizeof(unsigned) * b->capacity, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && !part.empty())
     e = cudaMemcpyAsync(part.data(), b->d_mass, sizeof(double) * part.size(), cudaMemcpyDeviceToHost, s);

@@ -8,7 +8,8 @@
 // (device.cuh: vectors of 2, 4 or 8 populations of one node that share the
 // sign of c_y), two ping-pong buffers in the caller's workspace.  The D = 3
 // sets store their z-even half.  One time step = one launch of k_step (or
-// k_step_z for D3Q216).
+// k_step_z for D3Q216, k_step_c for compensated storage); small solves run many
+// steps in one launch of k_steps_small.
 //
 // k_step mapping: a warp owns a strip of 32 consecutive x-nodes (the two
 // outer lanes on each side are halo lanes that load but do not store) and
