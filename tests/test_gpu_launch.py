@@ -204,3 +204,36 @@ def test_fields_of_many_admissions_arrive_whole(capacity, count, ny_hi):
         three.add_many(params, bad)
     assert "node 6 " in str(err.value)
     assert three.pool_free()[1] >= pool  # nothing was kept
+
+
+@pytest.mark.parametrize("nx,ny,nroots", [(4, 64, 4), (4, 200, 6), (40, 50, 4)])
+def test_a_whole_pass_replays_from_a_captured_graph(nx, ny, nroots):
+    """Initialisation, steps (on chip for few columns, an odd number of them),
+    moments and state as the nodes of one graph: each replay gives the bits of
+    the same calls made directly."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    prob = I.Problem(name="pass", nroots=nroots, nx=nx, ny=ny, bc_y=I.DIFFUSE, kn=0.1, b=-0.5, scheme=I.SPLIT,
+                     wall_ux=(-0.05, 0.05))
+    p = L.params_from_problem(prob)
+    fields = torch.from_numpy(I.random_fields(prob, amp_u=0.02, amp_T=0.02, amp_rho=0.02, seed=2)).cuda()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        direct, graphed = L.Solver(p, stream=side), L.Solver(p, stream=side)
+        direct.reinit(fields)
+        direct.step(9)
+        want = direct.moments(), direct.populations()
+    side.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        graphed.reinit(fields)
+        graphed.step(9)
+        got = graphed.moments(), graphed.populations()
+    for _ in range(3):
+        for t in got:
+            t.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
