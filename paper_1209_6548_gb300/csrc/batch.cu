@@ -91,13 +91,14 @@ struct InstRegs {
 };
 
 // The coefficients of a lane group in shared memory, 16-byte entries: the
-// advection's pair operands, NR of {kx, kx, -ax, -ax} (ix), NR/2 of
-// {ky, ky', -ay, -ay'} (the pair iy, iy + 1, iy even) and NR/2 of {-ay, -ay'}
-// for the x-sweep's input (0 in the printed update, whose x-fluxes take f^n
-// itself), then the scalars of InstRegs in two, {ny, walls, 0, instance} and
-// {output pointer, rows, first row}.
+// advection's pair operands, NR of {kx, kx, -ax, -ax} (ix) and NR/2 of
+// {ky, ky', -ay, -ay'} (the pair iy, iy + 1, iy even), then the scalars of
+// InstRegs in two, {ny, walls, split, instance} and {output pointer, rows,
+// first row}.
 template <int NR>
-constexpr int kCoefs = 2 * NR + 4;
+constexpr int kCoefScalars = NR + NR / 2;  // entry of the scalars
+template <int NR>
+constexpr int kCoefs = kCoefScalars<NR> + 4;
 
 template <int NR, class S = float, int NZ = 1>
 constexpr size_t kBatchRingBytes =
@@ -177,15 +178,12 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
     } else if (c < NR + NR / 2) {
       const int iy = 2 * (c - NR);
       v = make_float4(D.ky[iy], D.ky[iy + 1], -D.ay[iy], -D.ay[iy + 1]);
-    } else if (c < 2 * NR) {
-      const int iy = 2 * (c - NR - NR / 2);
-      v = D.split ? make_float4(-D.ay[iy], -D.ay[iy + 1], 0.f, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
-    } else if (c == 2 * NR) {
+    } else if (c == kCoefScalars<NR>) {
       v = make_float4(D.c_omega, D.visc_pow, D.b, D.beta);
-    } else if (c == 2 * NR + 1) {
+    } else if (c == kCoefScalars<NR> + 1) {
       v = make_float4(D.dtgx, D.dtgy, __int_as_float(D.vmode), __int_as_float(D.has_force));
-    } else if (c == 2 * NR + 2) {
-      v = make_float4(__int_as_float(ny), __int_as_float(walls), 0.f, __int_as_float(wi.inst));
+    } else if (c == kCoefScalars<NR> + 2) {
+      v = make_float4(__int_as_float(ny), __int_as_float(walls), __int_as_float(D.split), __int_as_float(wi.inst));
     } else {
       const unsigned long long o = reinterpret_cast<unsigned long long>(D.f[par ^ 1]);
       v = make_float4(__int_as_float((int)(unsigned)o), __int_as_float((int)(unsigned)(o >> 32)),
@@ -234,8 +232,8 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
   using T = typename Raw<Lay::VB>::T;
   T *ring = reinterpret_cast<T *>(smem_raw) + (size_t)(threadIdx.x >> 5) * kBRing * G * 32 + lane;
   int r1 = map_row(y0 + 1, ny, walls), r2 = map_row(y0 + 2, ny, walls);
-  const int4 *iflags = reinterpret_cast<const int4 *>(coef + (2 * NR + 2) * GPW);
-  const int4 *iout = reinterpret_cast<const int4 *>(coef + (2 * NR + 3) * GPW);
+  const int4 *iflags = reinterpret_cast<const int4 *>(coef + (kCoefScalars<NR> + 2) * GPW);
+  const int4 *iout = reinterpret_cast<const int4 *>(coef + (kCoefScalars<NR> + 3) * GPW);
   auto issue_rowload = [&](int k) {
     if (k < nrows) {
       const int2 fl = *reinterpret_cast<const int2 *>(iflags);  // ny, walls
@@ -264,7 +262,7 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
     float acc[Q];
     float omw;
     {
-      const float4 p = coef[2 * NR * GPW], q = coef[(2 * NR + 1) * GPW];
+      const float4 p = coef[kCoefScalars<NR> * GPW], q = coef[(kCoefScalars<NR> + 1) * GPW];
       const InstRegs P{p.x, p.y, p.z, p.w, q.x, q.y, __float_as_int(q.z), __float_as_int(q.w)};
       collide_any<NR, N>(fc, acc, omw, B.lat, P);
     }
@@ -272,11 +270,15 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
     const GroupLanes nb{srcL, srcR};
     const float2 omw2 = make_float2(omw, omw);
     const int4 fl = *iflags;
+    // the printed update's x-fluxes take f^n itself: a selection, since a zero
+    // coefficient would turn an infinite y-flux into NaN (0 Inf) there (it was
+    // that, 512 channels: D2Q16 13.3 us per step, now 13.5, D2Q36 41.7 -> 42.4,
+    // D3Q64 28.9 -> 30.3)
+    const bool split = fl.z != 0;
 #pragma unroll
     for (int a = 0; a < Q; a += 2) {  // packed pairs a, a+1 (same ix)
       const int iy = a % NR;
       const float4 cy = coef[(NR + iy / 2) * GPW];
-      const float2 nays = *reinterpret_cast<const float2 *>(coef + (NR + NR / 2 + iy / 2) * GPW);
       const float2 ky = make_float2(cy.x, cy.y), nay = make_float2(cy.z, cy.w);
       if ((iy >= H) != (iy + 1 >= H)) {  // a pair across c_y = 0 (D2Q36): one at a time
 #pragma unroll
@@ -284,18 +286,18 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
           float f0;
           const float diff = yflux(b % NR >= H, b, fc, s0, s1, ld, b == a ? ky.x : ky.y, f0);
           acc[b] = fmaf(omw, f0, fmaf(b == a ? nay.x : nay.y, diff, acc[b]));
-          xs[b] = fmaf(b == a ? nays.x : nays.y, diff, f0);
+          xs[b] = split ? fmaf(b == a ? nay.x : nay.y, diff, f0) : f0;
         }
         continue;
       }
       float2 f0;
       const float2 diff = yflux2(iy >= H, a, fc, s0, s1, ld, ky, f0);
       const float2 ac = fma2(omw2, f0, fma2(nay, diff, make_float2(acc[a], acc[a + 1])));
-      const float2 x2 = fma2(nays, diff, f0);
+      const float2 x2 = fma2(nay, diff, f0);
       acc[a] = ac.x;
       acc[a + 1] = ac.y;
-      xs[a] = x2.x;
-      xs[a + 1] = x2.y;
+      xs[a] = split ? x2.x : f0.x;
+      xs[a + 1] = split ? x2.y : f0.y;
     }
 #pragma unroll
     for (int ix = 0; ix < NR; ++ix) {

@@ -400,3 +400,37 @@ def test_d3q64_slots_with_every_wall_model_equal_alone():
         assert bt.info(sl).steps_done == n and bt.info(sl).q == 32
         assert bool((bt.populations(sl) == ref.populations()).all()), (q.storage, q.wall_T_amp, q.wall_specular)
         ref.close()
+
+
+@pytest.mark.parametrize("nroots,dim", [(4, 2), (6, 2), (4, 3)])
+@pytest.mark.parametrize("scheme", [I.UNSPLIT, I.SPLIT])
+def test_values_that_overflow_spread_as_in_the_solve_alone(nroots, dim, scheme):
+    """A slot whose fluxes overflow: which values turn infinite or NaN in each
+    step is the single-domain solver's pattern, value for value (the printed
+    update's x-fluxes take f^n, whatever the y-fluxes are)."""
+    import torch
+    prob = I.Problem(name="big", nx=4, ny=24, nroots=nroots, dim=dim, kn=0.1, b=-0.5, scheme=scheme, wall_ux=(0.0, 0.05))
+    p = L.params_from_problem(prob)
+    bt = L.Batch(capacity=1, nx=4, pool_bytes=pool_for([prob]))
+    bt.set_resident(False)
+    slot = bt.add(p)
+    raw, _ = bt.checkpoint(slot)
+    big = raw.view(torch.float32)
+    third = big.numel() // 3
+    big[third:2 * third:89] = 3.0e38
+    big[third + 40:2 * third:89] = -3.0e38
+    bt.resume(slot, raw, 0)
+    ref = L.Solver(p)
+    ref.set_populations(bt.populations(slot), 0)
+
+    def pattern(t):
+        return torch.nan_to_num(t, nan=1.5, posinf=2.5, neginf=-2.5)
+
+    seen = 0
+    for n in (1, 1, 3):
+        bt.step(n)
+        ref.step(n)
+        a, b = bt.populations(slot), ref.populations()
+        seen += int((~torch.isfinite(b)).sum())
+        assert torch.equal(pattern(a), pattern(b))
+    assert seen > 0
