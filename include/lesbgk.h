@@ -269,6 +269,13 @@ int lesbgk_set_launch(lesbgk *h, int32_t cells_per_thread, int32_t rows_per_segm
 /* Fill *out with the solver's time step, spacing and launch shape. */
 int lesbgk_get_info(const lesbgk *h, lesbgk_info *out);
 
+/* How lesbgk_step would take nsteps steps on this stream: *ctas is the size of
+ * the thread-block cluster that holds the whole solve on chip for many steps
+ * per launch (small FP32 solves, three or more steps in the call), 0 for one
+ * launch per step.  Results are bitwise the same either way.  A stream of a
+ * green context (a part of the device) takes one launch per step. */
+int lesbgk_on_chip_ctas(const lesbgk *h, int64_t nsteps, void *stream, int32_t *ctas);
+
 /* Release the handle (not the caller's workspace).  NULL is a no-op. */
 int lesbgk_destroy(lesbgk *h);
 

@@ -1720,13 +1720,36 @@ int pick_small(const lesbgk *h) {
   return best;
 }
 
-// nsteps steps of a small solve in place, in launches of at most kSmallSteps
-// (a few milliseconds each).
 constexpr int64_t kSmallSteps = 4096, kSmallFrom = 3;
-cudaError_t launch_small(lesbgk *h, int64_t nsteps, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  const int ctas = h->small_ctas;
-  for (int64_t done = 0; done < nsteps && e == cudaSuccess;) {
+
+// Whether the stream runs on a part of the device (a green context's): a
+// cluster chosen for the whole device may have no room there.
+bool on_part_of_device(cudaStream_t s) {
+  using Fn = int (*)(cudaStream_t, void **);
+  static const Fn get = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &f, 12040, cudaEnableDefault, &q);
+    cudaGetLastError();
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Fn>(f) : nullptr;
+  }();
+  void *green = nullptr;
+  return get && get(s, &green) == 0 && green;
+}
+
+// CTAs of the cluster that a call of nsteps steps on this stream runs in, 0
+// where it takes one launch per step.
+int small_ctas_for(const lesbgk *h, int64_t nsteps, cudaStream_t s) {
+  if (!h->small_ctas || h->rows_set || nsteps < kSmallFrom) return 0;
+  return h->small_ctas > 1 && on_part_of_device(s) ? 0 : h->small_ctas;
+}
+
+// Up to nsteps steps of a small solve in place, in launches of at most
+// kSmallSteps (a few milliseconds each); returns the steps launched, fewer
+// where a launch is refused.
+int64_t launch_small(lesbgk *h, int ctas, int64_t nsteps, cudaStream_t s) {
+  int64_t done = 0;
+  while (done < nsteps) {
     const int n = (int)(nsteps - done < kSmallSteps ? nsteps - done : kSmallSteps);
     cudaLaunchAttribute at[2] = {cluster_of(ctas), {}};
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1735,10 +1758,15 @@ cudaError_t launch_small(lesbgk *h, int64_t nsteps, cudaStream_t s) {
     c.stream = s;
     c.attrs = at;
     c.numAttrs = 2;
+    cudaError_t e = cudaSuccess;
     with_small(h, [&](auto kernel) { e = cudaLaunchKernelEx(&c, kernel, h->buf[h->cur], n, ctas, h->args); });
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // (an error of the context itself stays and is reported by the caller)
+      break;
+    }
     done += n;
   }
-  return e;
+  return done;
 }
 
 unsigned grid_for(const lesbgk *h, long long cells) {
@@ -1934,11 +1962,10 @@ extern "C" int lesbgk_step(lesbgk *h, int64_t nsteps, void *stream) {
   if (!h) return fail(LESBGK_EINVAL, "handle is NULL");
   if (nsteps < 0) return fail(LESBGK_EINVAL, "nsteps < 0");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (h->small_ctas && !h->rows_set && nsteps >= kSmallFrom) {
-    cudaError_t e = launch_small(h, nsteps, s);
-    if (e != cudaSuccess) return cuda_fail(e, "step kernel");
-    h->steps += nsteps;
-    return 0;
+  if (const int ctas = small_ctas_for(h, nsteps, s)) {
+    const int64_t done = launch_small(h, ctas, nsteps, s);
+    h->steps += done;
+    nsteps -= done;  // what a refused launch leaves takes one launch per step
   }
   for (int64_t k = 0; k < nsteps; ++k) {
     h->args.seed = (unsigned)(h->steps + k) * 0x9e3779b9u + 0x7f4a7c15u;  // a new rounding key per step
@@ -2162,6 +2189,12 @@ extern "C" int lesbgk_get_info(const lesbgk *h, lesbgk_info *out) {
   out->order = h->order;
   out->cells_per_thread = h->cpt;
   out->rows_per_segment = h->rows;
+  return 0;
+}
+
+extern "C" int lesbgk_on_chip_ctas(const lesbgk *h, int64_t nsteps, void *stream, int32_t *ctas) {
+  if (!h || !ctas) return fail(LESBGK_EINVAL, "NULL argument");
+  *ctas = small_ctas_for(h, nsteps, static_cast<cudaStream_t>(stream));
   return 0;
 }
 

@@ -37,7 +37,7 @@ SYMBOLS = ("lesbgk_workspace_size", "lesbgk_create", "lesbgk_reinit", "lesbgk_st
            "lesbgk_batch_autotune", "lesbgk_batch_pool_free", "lesbgk_batch_destroy", "lesbgk_batch_add_many",
            "lesbgk_batch_moments_many", "lesbgk_batch_set_resident", "lesbgk_batch_get_launch",
            "lesbgk_batch_check_guards", "lesbgk_batch_debug_poison", "lesbgk_batch_raw_bytes",
-           "lesbgk_batch_get_raw", "lesbgk_batch_set_raw")
+           "lesbgk_batch_get_raw", "lesbgk_batch_set_raw", "lesbgk_on_chip_ctas")
 
 
 class Params(C.Structure):
@@ -93,6 +93,7 @@ def lib():
             L.lesbgk_set_populations.argtypes = [vp, vp, i64, vp]
             L.lesbgk_set_launch.argtypes = [vp, C.c_int32, C.c_int32]
             L.lesbgk_get_info.argtypes = [vp, C.POINTER(Info)]
+            L.lesbgk_on_chip_ctas.argtypes = [vp, i64, vp, C.POINTER(C.c_int32)]
             L.lesbgk_destroy.argtypes = [vp]
             L.lesbgk_moments_noalloc.argtypes = [C.POINTER(Params), vp, vp, vp, vp]
             L.lesbgk_rows_bytes.argtypes = [vp, C.c_int32, C.POINTER(C.c_size_t)]
@@ -314,6 +315,13 @@ class Solver:
 
     def set_launch(self, cells_per_thread: int = 0, rows_per_segment: int = 0) -> None:
         set_launch(self.handle, cells_per_thread, rows_per_segment)
+
+    def on_chip_ctas(self, n: int) -> int:
+        """Thread blocks of the cluster that step(n) keeps the solve in, 0 for one launch per step."""
+        out = C.c_int32()
+        _check(lib().lesbgk_on_chip_ctas(C.c_void_p(self.handle), C.c_int64(n), C.c_void_p(self.stream.cuda_stream),
+                                         C.byref(out)))
+        return out.value
 
     @property
     def info(self) -> Info:

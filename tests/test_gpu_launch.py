@@ -237,3 +237,83 @@ def test_a_whole_pass_replays_from_a_captured_graph(nx, ny, nroots):
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+class _PartOfTheDevice:
+    """A stream of a green context that holds the fewest SMs the driver gives."""
+
+    def __enter__(self):
+        import ctypes as C
+        import torch
+
+        class Resource(C.Structure):  # CUdevResource: type, padding, SM counts
+            _fields_ = [("type", C.c_int), ("pad", C.c_ubyte * 92), ("sms", C.c_uint), ("rest", C.c_ubyte * 44)]
+
+        torch.zeros(1, device="cuda")
+        self.cu = C.CDLL("libcuda.so.1")
+
+        def call(name, *args):
+            rc = getattr(self.cu, name)(*args)
+            if rc:
+                pytest.skip(f"{name}: error {rc}")
+
+        whole, part, rest = Resource(), Resource(), Resource()
+        call("cuDeviceGetDevResource", C.c_int(torch.cuda.current_device()), C.byref(whole), C.c_int(1))
+        groups = C.c_uint(1)
+        call("cuDevSmResourceSplitByCount", C.byref(part), C.byref(groups), C.byref(whole), C.byref(rest), C.c_uint(0),
+             C.c_uint(8))
+        desc, self.green, self.handle = C.c_void_p(), C.c_void_p(), C.c_void_p()
+        call("cuDevResourceGenerateDesc", C.byref(desc), C.byref(part), C.c_uint(1))
+        call("cuGreenCtxCreate", C.byref(self.green), desc, C.c_int(torch.cuda.current_device()), C.c_uint(1))
+        call("cuGreenCtxStreamCreate", C.byref(self.handle), self.green, C.c_uint(1), C.c_int(0))
+        self.sms, self.all_sms = part.sms, whole.sms
+        return self
+
+    def __exit__(self, *exc):
+        self.cu.cuStreamSynchronize(self.handle)
+        self.cu.cuStreamDestroy_v2(self.handle)
+        self.cu.cuGreenCtxDestroy(self.green)
+
+
+def test_small_solves_march_on_a_part_of_the_device():
+    """The cluster of an on-chip solve is chosen for the whole device; on a
+    stream that has a part of it the call takes one launch per step, with the
+    same bits."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    p = L.params_from_problem(I.Problem(name="part", nx=4, ny=1000, bc_y=I.DIFFUSE, kn=0.1, b=-0.5, wall_ux=(0.0, 0.05)))
+    whole = L.Solver(p)
+    whole.step(9)
+    torch.cuda.synchronize()
+    assert whole.on_chip_ctas(9) == 16
+    with _PartOfTheDevice() as part:
+        assert 0 < part.sms < part.all_sms
+        s = L.Solver(p)
+        torch.cuda.synchronize()
+        s.stream = torch.cuda.ExternalStream(part.handle.value)
+        assert s.on_chip_ctas(9) == 0
+        s.step(9)
+        got = s.populations()
+        s.stream.synchronize()
+        assert s.info.steps_done == 9 and torch.equal(got, whole.populations())
+
+
+def test_which_calls_keep_the_solve_on_chip():
+    """Three or more steps of FP32 solves on up to 32 periodic columns, at one
+    node per thread of at most 16 blocks, with steady walls and no rows set."""
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    def ctas(n=3, rows=0, storage=0, **kw):
+        p = L.params_from_problem(I.Problem(name="path", **{**dict(nx=4, ny=64, bc_y=I.DIFFUSE, kn=0.1, b=-0.5), **kw}))
+        p.storage = storage
+        s = L.Solver(p)
+        if rows:
+            s.set_launch(0, rows)
+        return s.on_chip_ctas(n)
+
+    assert ctas() > 0 and ctas(ny=1000) == 16 and ctas(nx=32, ny=128) == 16
+    assert ctas(nroots=6) > 0 and ctas(dim=3) > 0 and ctas(bc_y=I.PERIODIC) > 0 and ctas(nx=1, ny=4) == 1
+    assert ctas(n=2) == 0 and ctas(rows=3) == 0 and ctas(nx=33, ny=20) == 0 and ctas(ny=3) == 0
+    assert ctas(storage=1) == 0 and ctas(storage=3) == 0 and ctas(nroots=6, dim=3) == 0
+    assert ctas(bc_x=I.DIFFUSE) == 0 and ctas(wall_T_amp=0.02, wall_T_freq=0.5) == 0 and ctas(nx=32, ny=4096) == 0
