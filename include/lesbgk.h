@@ -375,6 +375,13 @@ int lesbgk_batch_set_resident(lesbgk_batch *b, int32_t on, int32_t steps_per_lau
 /* The launch configuration in use (any pointer may be NULL). */
 int lesbgk_batch_get_launch(const lesbgk_batch *b, int32_t *rows, int32_t *resident, int32_t *steps_per_launch,
                             int32_t *resident_max_ny);
+/* The work list as it stands for one slot (any pointer may be NULL; rebuilds the
+ * list on the stream where solves came or went): the rows of its step items (0:
+ * the resident kernel holds it), the chains its class's solves are dealt to, and
+ * the rows of the items by which residuals and moments read it (of several
+ * items, the longest). */
+int lesbgk_batch_get_work(lesbgk_batch *b, int32_t slot, int32_t *step_rows, int32_t *chains, int32_t *read_rows,
+                          void *stream);
 /* Autotuner: time a 64-step chunk of the current slots for each candidate
  * rows per work item, each with the resident kernel off, and on at 16 and 64
  * steps per launch for instances of at most 64, 128, 256 rows or as many as

@@ -1751,6 +1751,26 @@ extern "C" int lesbgk_batch_get_launch(const lesbgk_batch *b, int32_t *rows, int
   return 0;
 }
 
+extern "C" int lesbgk_batch_get_work(lesbgk_batch *b, int32_t slot, int32_t *step_rows, int32_t *chains,
+                                     int32_t *read_rows, void *stream) {
+  if (!b || slot < 0 || slot >= b->capacity || !b->slots[slot].used) return fail(LESBGK_EINVAL, "no such slot");
+  if (int rc = ensure_items(b, static_cast<cudaStream_t>(stream))) return rc;
+  const int cls = b->slots[slot].cls;
+  auto longest = [&](const int (&range)[2]) {  // the slot's longest item of a range
+    int rows = 0;
+    for (int k = range[0]; k < range[0] + range[1]; ++k)
+      if (b->items[k].inst == slot) rows = std::max(rows, b->items[k].rows);
+    return rows;
+  };
+  if (step_rows) *step_rows = longest(b->range[cls]);
+  if (read_rows) *read_rows = longest(b->range_all[cls]);
+  if (chains) {
+    *chains = 0;
+    for (const auto &c : b->range_chain[cls]) *chains += c[1] > 0;
+  }
+  return 0;
+}
+
 extern "C" int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates, int32_t n, int32_t *chosen,
                                      void *stream) {
   lesbgk_internal::Range range_("lesbgk_batch_autotune");

@@ -37,7 +37,7 @@ SYMBOLS = ("lesbgk_workspace_size", "lesbgk_create", "lesbgk_reinit", "lesbgk_st
            "lesbgk_batch_autotune", "lesbgk_batch_pool_free", "lesbgk_batch_destroy", "lesbgk_batch_add_many",
            "lesbgk_batch_moments_many", "lesbgk_batch_set_resident", "lesbgk_batch_get_launch",
            "lesbgk_batch_check_guards", "lesbgk_batch_debug_poison", "lesbgk_batch_raw_bytes",
-           "lesbgk_batch_get_raw", "lesbgk_batch_set_raw", "lesbgk_on_chip_ctas")
+           "lesbgk_batch_get_raw", "lesbgk_batch_set_raw", "lesbgk_on_chip_ctas", "lesbgk_batch_get_work")
 
 
 class Params(C.Structure):
@@ -110,6 +110,7 @@ def lib():
             L.lesbgk_batch_moments_many.argtypes = [vp, i32, vp, vp, vp]
             L.lesbgk_batch_set_resident.argtypes = [vp, i32, i32, i32, vp]
             L.lesbgk_batch_get_launch.argtypes = [vp, vp, vp, vp, vp]
+            L.lesbgk_batch_get_work.argtypes = [vp, i32, vp, vp, vp, vp]
             L.lesbgk_batch_step.argtypes = [vp, i64, vp]
             L.lesbgk_batch_residuals.argtypes = [vp, vp, vp, vp]
             L.lesbgk_residual.argtypes = [vp, vp, i64, vp, vp, vp]
@@ -481,6 +482,13 @@ class Batch:
         _check(lib().lesbgk_batch_get_launch(C.c_void_p(self.handle), *[C.byref(x) for x in v]))
         return {"rows_per_item": v[0].value, "resident": bool(v[1].value), "steps_per_launch": v[2].value,
                 "resident_max_ny": v[3].value}
+
+    def work(self, slot: int) -> dict:
+        """The work list for one slot: rows per step item (0: resident), chains of its class, rows
+        per item of residuals and moments."""
+        v = [C.c_int32() for _ in range(3)]
+        _check(lib().lesbgk_batch_get_work(C.c_void_p(self.handle), C.c_int32(slot), *[C.byref(x) for x in v], self._s))
+        return {"step_rows": v[0].value, "chains": v[1].value, "read_rows": v[2].value}
 
     def check_guards(self):
         """Per slot: 1 where the guard words after the slot's memory changed

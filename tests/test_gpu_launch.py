@@ -317,3 +317,90 @@ def test_which_calls_keep_the_solve_on_chip():
     assert ctas(n=2) == 0 and ctas(rows=3) == 0 and ctas(nx=33, ny=20) == 0 and ctas(ny=3) == 0
     assert ctas(storage=1) == 0 and ctas(storage=3) == 0 and ctas(nroots=6, dim=3) == 0
     assert ctas(bc_x=I.DIFFUSE) == 0 and ctas(wall_T_amp=0.02, wall_T_freq=0.5) == 0 and ctas(nx=32, ny=4096) == 0
+
+
+def _batch(probs, storage=(0,), **kw):
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    params = [L.params_from_problem(p) for p in probs]
+    for k, p in enumerate(params):
+        if p.wall_specular == 0.0:
+            p.storage = storage[k % len(storage)]
+    bt = L.Batch(capacity=len(params), nx=probs[0].nx, pool_bytes=sum(L.batch_slot_bytes(p) for p in params) + (1 << 20))
+    for name, value in kw.items():
+        getattr(bt, name)(value)
+    return bt, params, bt.add_many(params)
+
+
+def test_which_work_items_a_batch_makes():
+    """One chain of short items for a small batch, four once the items fill the
+    chip, the resident kernel for short solves alone; reads in 32-row items."""
+    bt, params, slots = _batch(I.batch_mix(n=150, seed=150, ny_lo=16, ny_hi=1024))
+    for s, p in zip(slots, params):
+        w = bt.work(s)
+        assert 1 <= w["step_rows"] <= min(64, p.ny) and w["chains"] == 4 and w["read_rows"] == min(32, p.ny)
+    bt, params, slots = _batch(I.batch_mix(n=40, seed=40, ny_lo=2, ny_hi=300))
+    assert all(bt.work(s)["chains"] == 1 and bt.work(s)["step_rows"] == 1 for s in slots)
+    bt, params, slots = _batch(I.batch_mix(n=20, seed=20, ny_lo=2, ny_hi=64))
+    for s, p in zip(slots, params):
+        assert bt.work(s) == {"step_rows": 0, "chains": 0, "read_rows": min(32, p.ny)}
+    bt.set_resident(False)
+    bt.set_rows(5)
+    assert all(bt.work(s)["step_rows"] == min(5, p.ny) == bt.work(s)["read_rows"] for s, p in zip(slots, params))
+
+
+@pytest.mark.parametrize("storage", [(1,), (0, 2)])
+def test_four_chains_keep_each_slots_clock(storage):
+    """16-bit rounding keys and heated walls follow a slot's own step count:
+    four chains against fixed rows, through graphs, single steps, removals and
+    re-admissions at another parity."""
+    import torch
+    from dataclasses import replace
+
+    probs = [replace(p, wall_T_amp=0.02, wall_T_freq=0.5) if k % 2 else p
+             for k, p in enumerate(I.batch_mix(n=300, seed=7, ny_lo=16, ny_hi=1024))]
+    got = []
+    for kw in ({}, {"set_resident": False, "set_rows": 32}):
+        bt, params, slots = _batch(probs, storage, **kw)
+        if not kw:
+            assert max(bt.work(s)["chains"] for s in slots) == 4
+        bt.step(64 + 3)
+        for k in range(0, 300, 5):
+            bt.remove(slots[k])
+        bt.step(1)
+        for k in range(0, 300, 10):
+            slots[k] = bt.add(params[k])
+        bt.step(64 + 5)
+        got.append([bt.populations(slots[k]) for k in range(300) if k % 5 or k % 10 == 0])
+        bt.close()
+    for a, b in zip(*got):
+        assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
+
+
+@pytest.mark.parametrize("storage", [0, 1])
+def test_steps_that_fill_the_chip_overlap_safely_with_other_work(storage):
+    """On a grid whose steps fill the chip even single-step calls overlap what
+    runs before them: foreign kernels, moments and state reads between."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    prob = I.Problem(name="fills", nx=1030, ny=1021, bc_y=I.DIFFUSE, kn=0.1, b=-0.5, scheme=I.SPLIT,
+                     wall_ux=(0.0, 0.05))
+    p = L.params_from_problem(prob)
+    p.storage = storage
+    init = I.random_fields(prob, seed=1)
+    many = L.Solver(p, h_init=init)
+    many.step(18)
+    blocks = 37 * -(-1021 // many.info.rows_per_segment) / 4  # 28 columns per warp, four warps per block
+    assert blocks >= 3.5 * torch.cuda.get_device_properties(0).multi_processor_count
+    single = L.Solver(p, h_init=init)
+    noise = torch.zeros(1 << 22, device="cuda")
+    for k in range(18):
+        if k % 3 == 0:
+            noise.add_(1.0)
+        single.step(1)
+        if k % 5 == 0:
+            single.moments()
+        if k % 7 == 0:
+            single.populations()
+    assert torch.equal(many.populations(), single.populations())
