@@ -988,7 +988,13 @@ void pick_rows(lesbgk_batch *b) {
   const double sms = b->sm_count > 0 ? b->sm_count : 152;
   const double per_block = (double)(kBBlock / b->W);  // items a block takes
   for (int cls = 0; cls < kNumClasses; ++cls) {
-    if (!(rows[cls] > 0.0)) continue;
+    if (!(rows[cls] > 0.0)) {  // no solve of it takes the per-step kernel: the reads go by the caller's rows
+      if (!b->auto_rows) {
+        b->rows_of[cls] = b->rows;
+        b->chains_of[cls] = 1;
+      }
+      continue;
+    }
     const double cap = (cls % 3 == 0 ? 4 : 2) * sms * work[cls] / all;
     int r = b->rows;
     if (b->auto_rows) r = (int)std::fmin(64.0, std::ceil(rows[cls] / (per_block * 1.5 * cap)));

@@ -404,3 +404,36 @@ def test_steps_that_fill_the_chip_overlap_safely_with_other_work(storage):
         if k % 7 == 0:
             single.populations()
     assert torch.equal(many.populations(), single.populations())
+
+
+def test_reads_of_resident_solves_go_by_the_callers_rows():
+    """Rows set by the caller hold for the reads of solves that the resident
+    kernel steps, whatever rows their class had before, and the reads give the
+    same bits."""
+    import numpy as np
+    import torch
+
+    probs = I.batch_mix(n=24, seed=3, ny_lo=16, ny_hi=64)
+    bt, params, slots = _batch(probs, set_resident=True)
+    other, _, slots2 = _batch(probs, set_resident=False)
+    other.set_rows(32)
+    other.set_rows(4)
+    other.set_resident(True)
+    for x in (bt, other):
+        x.set_rows(32)
+    for s, t, p in zip(slots, slots2, params):
+        assert bt.work(s) == other.work(t) == {"step_rows": 0, "chains": 0, "read_rows": min(32, p.ny)}
+    free, _, slots3 = _batch(probs)  # the rules: items of 32 rows
+    for x in (bt, other, free):
+        x.step(64)
+    first = [x.residuals(mass=True)[1] for x in (bt, other, free)]
+    for x in (bt, other, free):
+        x.step(64)
+    second = [x.residuals(mass=True) for x in (bt, other, free)]
+    for m, (r, m2) in zip(first[1:], second[1:]):
+        assert np.array_equal(m, first[0]) and np.array_equal(r, second[0][0]) and np.array_equal(m2, second[0][1])
+    outs = [[torch.empty((9, p.ny, 4), device="cuda") for p in params] for _ in range(3)]
+    for x, sl, o in zip((bt, other, free), (slots, slots2, slots3), outs):
+        x.moments_many(sl, o)
+    for a, b, c in zip(*outs):
+        assert torch.equal(a, b) and torch.equal(a, c)
