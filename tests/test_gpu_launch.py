@@ -437,3 +437,28 @@ def test_reads_of_resident_solves_go_by_the_callers_rows():
         x.moments_many(sl, o)
     for a, b, c in zip(*outs):
         assert torch.equal(a, b) and torch.equal(a, c)
+
+
+@pytest.mark.parametrize("ny", [4, 5, 6, 7, 33])
+def test_a_bad_field_is_found_at_its_node(ny):
+    """The check of a batched solve's fields names the first bad node wherever
+    it lies among the lanes of the check, and takes huge finite values."""
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    prob = I.Problem(name="bad", nx=1, ny=ny, bc_y=I.DIFFUSE, kn=0.1, b=-0.5)
+    p = L.params_from_problem(prob)
+    bt = L.Batch(capacity=2, nx=1, pool_bytes=4 * L.batch_slot_bytes(p))
+    rest = np.zeros((4, ny, 1))
+    rest[0] = rest[3] = 1.0
+    for field, value in ((0, 0.0), (0, -1.0), (0, np.nan), (0, np.inf), (1, np.nan), (1, -np.inf), (2, np.inf), (3, 0.0),
+                         (3, np.nan), (3, np.inf)):
+        for node in {0, 1, ny // 2, ny - 2, ny - 1}:
+            f = rest.copy()
+            f[field, node:, 0] = value
+            f[2, ny - 1, 0] = np.inf  # a later one is not named
+            with pytest.raises(L.LesbgkError) as err:
+                bt.add(p, f)
+            assert f"node {node} " in str(err.value)
+    f = rest.copy()
+    f[1, :, 0], f[2, :, 0] = 1.5e308, 1.5e308
+    bt.remove(bt.add(p, f))  # finite, though their sum is not
