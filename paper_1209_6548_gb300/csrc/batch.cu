@@ -20,6 +20,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -782,13 +783,15 @@ struct lesbgk_batch {
   int range_chain[kNumClasses][kChains][2] = {};
   int graph_grid[kNumClasses][kChains] = {};
   bool graph_dirty = true;
-  std::vector<double> stage;  // fields on their way to the device (lesbgk_batch_add_many)
+  std::unique_ptr<double[]> stage;  // fields on their way to the device (lesbgk_batch_add_many)
+  size_t stage_doubles = 0;
   bool items_dirty = false;  // slots changed since the work list was uploaded
 };
 
 namespace {
 
 constexpr size_t kStageDoubles = 1 << 20;  // at most 8 MB of fields staged at a time
+constexpr size_t kStagedMost = 20480;      // doubles of the largest fields that are staged (160 kB)
 constexpr size_t kItemsPerSlot = 1024;  // work-list room: items per slot (rows/8 for ny <= 8192)
 
 struct Layout0 {
@@ -1444,22 +1447,39 @@ extern "C" int lesbgk_batch_add_many(lesbgk_batch *b, int32_t n, const lesbgk_pa
     // (slots in the range not taken here keep their device descriptors: copy
     // them back unchanged from the host mirror, which is the same data)
     e = cudaMemcpyAsync(b->d_desc + lo, desc.data(), sizeof(InstDesc) * desc.size(), cudaMemcpyHostToDevice, s);
-    // The fields class by class through one staging area, copied and
-    // initialised whenever it is full (512 channels: 4.2 ms with a copy per slot,
-    // 3.1 ms staged, checks included); a solve too large for it goes to its own
-    // spare buffer.  The area is the residual pass's per-item scratch: that
-    // call returns only after its work is done, so nothing in flight uses it.
+    // Small fields go class by class through one staging area, copied and
+    // initialised whenever it is full (512 channels: 5.9 ms with a copy per solve,
+    // 3.2 ms staged, checks included).  Fields of which the area holds few, or
+    // of more than 160 kB, go straight to the solve's own spare buffer, copied by
+    // the host once less and initialised side by side: 512 solves (us, direct
+    // against staged) 8.8 and 6.9 ms at 96 kB, 10.6 and 10.6 at 160, 14.3 and 18.6
+    // at 256; 64 solves in room for one at a time, 512 kB, 3.2 and 10.8 ms.
+    // The area is the residual pass's per-item scratch: that call returns only
+    // after its work is done, so nothing in flight uses it.
     double *const d_stage = b->d_mass;
     const size_t room = std::min<size_t>((size_t)b->capacity * kItemsPerSlot, kStageDoubles);
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
     std::stable_sort(order.begin(), order.end(),
                      [&](int x, int y) { return b->slots[taken[x]].cls < b->slots[taken[y]].cls; });
+    const size_t most = n < 4 ? 0 : std::min(room / 16, kStagedMost);
+    auto staged = [&](int i) {  // doubles of fields i to stage, 0 for none
+      const size_t count = 4 * (size_t)ps[i].nx * ps[i].ny;
+      return h_inits && h_inits[i] && count <= most ? count : 0;
+    };
+    size_t need = 0;
+    for (int i = 0; i < n; ++i) need += staged(i);
+    need = std::min(need, room);
+    if (need > b->stage_doubles) {
+      b->stage_doubles = 0;
+      b->stage.reset(new (std::nothrow) double[need]);
+      if (b->stage) b->stage_doubles = need;
+    }
     std::vector<InitItem> list;
     size_t used = 0, begin = 0;  // doubles staged; first entry of order not yet initialised
     auto flush = [&](size_t end) {
       if (e == cudaSuccess && used)
-        e = cudaMemcpyAsync(d_stage, b->stage.data(), used * sizeof(double), cudaMemcpyHostToDevice, s);
+        e = cudaMemcpyAsync(d_stage, b->stage.get(), used * sizeof(double), cudaMemcpyHostToDevice, s);
       if (e == cudaSuccess && !list.empty())
         e = cudaMemcpyAsync(b->d_list, list.data(), sizeof(InitItem) * list.size(), cudaMemcpyHostToDevice, s);
       for (size_t k = begin; k < end && e == cudaSuccess;) {
@@ -1491,13 +1511,12 @@ extern "C" int lesbgk_batch_add_many(lesbgk_batch *b, int32_t n, const lesbgk_pa
       const size_t count = 4 * (size_t)sl.p.nx * sl.p.ny;
       if (!fields) {
         list.push_back({taken[i], -2});
-      } else if (count > room) {
+      } else if (!staged(i) || !b->stage_doubles) {
         e = cudaMemcpyAsync(sl.desc.f[b->par ^ 1], fields, count * sizeof(double), cudaMemcpyHostToDevice, s);
         list.push_back({taken[i], -1});
       } else {
-        if (used + count > room) flush(k);
-        if (b->stage.size() < used + count) b->stage.resize(std::min(room, std::max(used + count, 2 * b->stage.size())));
-        std::memcpy(b->stage.data() + used, fields, count * sizeof(double));
+        if (used + count > b->stage_doubles) flush(k);
+        std::memcpy(b->stage.get() + used, fields, count * sizeof(double));
         list.push_back({taken[i], (int)used});
         used += count;
       }

@@ -462,3 +462,39 @@ def test_a_bad_field_is_found_at_its_node(ny):
     f = rest.copy()
     f[1, :, 0], f[2, :, 0] = 1.5e308, 1.5e308
     bt.remove(bt.add(p, f))  # finite, though their sum is not
+
+
+@pytest.mark.parametrize("capacity,sizes", [
+    (3, (40, 40, 700)),                      # three solves: straight to their buffers
+    (16, (31, 32, 33, 64, 100, 255, 256)),   # staging room 16 kdoubles: staged up to 1024 of them, 8 rows of 32 columns
+    (512, (159, 160, 161, 8, 1200, 700, 64)),  # staged up to 160 kB: 160 rows
+])
+@pytest.mark.parametrize("pinned", [False, True])
+def test_large_and_pinned_fields_arrive_whole(capacity, sizes, pinned):
+    """Fields on both sides of the size from which they go straight to the
+    solve's own buffer, in one call, repeated: the populations of single
+    admissions, bitwise."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    probs = [I.Problem(name="f", nx=32, ny=ny, nroots=6 if k % 3 == 2 else 4, bc_y=I.DIFFUSE, kn=0.1, b=-0.5)
+             for k, ny in enumerate(sizes * 2)]
+    if capacity == 16:
+        probs = [I.Problem(name="f", nx=32, ny=ny, bc_y=I.DIFFUSE, kn=0.1, b=-0.5) for ny in (7, 8, 9, *sizes)]
+    if capacity == 3:
+        probs = probs[:3]
+    params = [L.params_from_problem(p) for p in probs]
+    fields = []
+    for k, p in enumerate(probs):
+        t = torch.from_numpy(I.random_fields(p, seed=k))
+        fields.append((t.pin_memory() if pinned else t).numpy())
+    pool = sum(L.batch_slot_bytes(p) for p in params)
+    many, one = (L.Batch(capacity=capacity, nx=32, pool_bytes=pool) for _ in range(2))
+    want = [one.populations(one.add(p, f)) for p, f in zip(params, fields)]
+    for _ in range(2):
+        slots = many.add_many(params, fields)
+        for s, w in zip(slots, want):
+            assert torch.equal(many.populations(s), w)
+        assert int(many.check_guards().sum()) == 0
+        for s in slots:
+            many.remove(s)
