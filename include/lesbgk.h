@@ -357,8 +357,9 @@ int lesbgk_batch_get_info(const lesbgk_batch *b, int32_t slot, lesbgk_info *out)
 int lesbgk_batch_raw_bytes(const lesbgk_batch *b, int32_t slot, size_t *bytes);
 int lesbgk_batch_get_raw(lesbgk_batch *b, int32_t slot, void *d_out, void *stream);
 int lesbgk_batch_set_raw(lesbgk_batch *b, int32_t slot, const void *d_in, int64_t steps_done, void *stream);
-/* Rows per work item; until it is set (or lesbgk_batch_autotune called) the
- * rows follow the solves in the batch.  Results do not depend on it. */
+/* Rows per work item; until it is set (or lesbgk_batch_autotune called), and
+ * again from lesbgk_batch_set_auto, the rows follow the solves in the batch.
+ * Results do not depend on it. */
 int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream);
 /* Resident kernel: D2Q16 FP32 instances of at most max_ny rows
  * (0 keeps the current limit, 128 by default) whose two population buffers
@@ -368,8 +369,9 @@ int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream);
  * per launch, while the other instances take one launch per step; in the
  * 64-step graphs the two run side by side.  A resident instance is one
  * block's serial work, so tall ones are better left to the per-step kernel:
- * until this call (or lesbgk_batch_autotune) it is on where every solve of
- * the batch has at most 64 rows, and off otherwise.
+ * until this call (or lesbgk_batch_autotune), and again from
+ * lesbgk_batch_set_auto, it is on where every solve of the batch has at most 64
+ * rows, and off otherwise.
  * Results do not depend on the choice (bitwise). */
 int lesbgk_batch_set_resident(lesbgk_batch *b, int32_t on, int32_t steps_per_launch, int32_t max_ny, void *stream);
 /* The launch configuration in use (any pointer may be NULL). */
@@ -382,13 +384,22 @@ int lesbgk_batch_get_launch(const lesbgk_batch *b, int32_t *rows, int32_t *resid
  * items, the longest). */
 int lesbgk_batch_get_work(lesbgk_batch *b, int32_t slot, int32_t *step_rows, int32_t *chains, int32_t *read_rows,
                           void *stream);
-/* Autotuner: time a 64-step chunk of the current slots for each candidate
- * rows per work item, each with the resident kernel off, and on at 16 and 64
- * steps per launch for instances of at most 64, 128, 256 rows or as many as
- * fit (the state is left unchanged: every timed launch writes the spare
- * buffers), and keep the fastest; *chosen receives its rows per item
- * (lesbgk_batch_get_launch gives the rest). */
+/* Rows per work item, chains and the resident kernel by the batch's contents,
+ * as it was created. */
+int lesbgk_batch_set_auto(lesbgk_batch *b, void *stream);
+/* Autotuner: time a 64-step chunk of the current slots, as the step graph that
+ * would run, for each candidate rows per work item, each with the resident
+ * kernel off, and on at 16 and 64 steps per launch for instances of at most 64,
+ * 128, 256 rows or as many as fit (the state is left unchanged: every timed
+ * launch writes the spare buffers), and keep the fastest; *chosen receives its
+ * rows per item (lesbgk_batch_get_launch gives the rest).  The choice is among
+ * the caller's rows: the batch's own rule may know better ones.  A call that
+ * fails leaves the configuration as it was. */
 int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates, int32_t n, int32_t *chosen, void *stream);
+/* The same with the rules of lesbgk_batch_set_auto as one more candidate;
+ * *chosen receives 0 where they win and are kept. */
+int lesbgk_batch_autotune_rules(lesbgk_batch *b, const int32_t *candidates, int32_t n, int32_t *chosen,
+                                void *stream);
 /* Largest free block and total free bytes of the pool. */
 int lesbgk_batch_pool_free(const lesbgk_batch *b, size_t *largest, size_t *total);
 /* Guard words (a check for writes outside a slot's memory; the paper has no

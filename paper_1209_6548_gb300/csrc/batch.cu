@@ -1121,15 +1121,16 @@ void drop_graph(lesbgk_batch *b) {
 // step (the classes step other instances: their chains are independent), each
 // step after the previous one; grids sized with head room for the
 // current work list (kernels read their item counts from device memory, so
-// the graph stays valid while slots come and go).
-int build_graph(lesbgk_batch *b) {
+// the graph stays valid while slots come and go).  `timing`: every launch reads
+// the current buffers and writes the spare ones, so the state stays as it is.
+int build_graph(lesbgk_batch *b, bool timing = false) {
   drop_graph(b);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaGraphCreate(&g, 0);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphCreate");
   std::vector<BatchArgs> args_store((size_t)kNumClasses * kChains);
   BatchArgs(*args)[kChains] = reinterpret_cast<BatchArgs(*)[kChains]>(args_store.data());
-  int pars[2] = {0, 1};
+  int pars[2] = {timing ? b->par : 0, timing ? b->par : 1};
   cudaGraphNode_t prev[kNumClasses][kChains] = {};
   cudaGraphEdgeData edge{};  // the next step may be scheduled while this one runs
   edge.from_port = cudaGraphKernelNodePortProgrammatic;
@@ -1164,7 +1165,7 @@ int build_graph(lesbgk_batch *b) {
   // independent of the per-step chain (they touch other instances)
   BatchArgs a0 = make_args(b, 0);
   const int *rl = b->d_rlist;
-  int K = b->resident_k, p0 = 0;
+  int K = b->resident_k, p_in = timing ? b->par : 0, p_out = timing ? b->par ^ 1 : 0;
   for (int k = 0; k < kBuckets && e == cudaSuccess; ++k) {
     const int n = b->rrange[k][1];
     b->graph_rgrid[k] = n ? n + n / 4 + 8 : 0;
@@ -1173,7 +1174,7 @@ int build_graph(lesbgk_batch *b) {
     cudaGraphNode_t last = nullptr;
     for (int c = 0; c < kGraphSteps / K && e == cudaSuccess; ++c) {
       cudaKernelNodeParams kp{};
-      void *kargs[] = {&a0, &rl, &rr, &K, &p0, &p0};
+      void *kargs[] = {&a0, &rl, &rr, &K, &p_in, &p_out};
       kp.func = resident_fn(b->W);
       kp.gridDim = dim3(b->graph_rgrid[k]);
       kp.blockDim = dim3(kBBlock);
@@ -1190,7 +1191,7 @@ int build_graph(lesbgk_batch *b) {
     b->graph = nullptr;
     return cuda_fail(e, "building the step graph");
   }
-  b->graph_dirty = false;
+  b->graph_dirty = timing;
   return 0;
 }
 
@@ -1736,11 +1737,21 @@ extern "C" int lesbgk_batch_get_info(const lesbgk_batch *b, int32_t slot, lesbgk
   return 0;
 }
 
-extern "C" int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream) {
-  if (!b || rows < 1 || rows > 4096) return fail(LESBGK_EINVAL, "rows must be in [1, 4096]");
+namespace {
+
+int check_rows(const lesbgk_batch *b, int rows) {
+  if (rows < 1 || rows > 4096) return fail(LESBGK_EINVAL, "rows must be in [1, 4096]");
   for (auto &sl : b->slots)
     if (sl.used && (long long)(sl.p.ny + rows - 1) / rows > (long long)kItemsPerSlot)
       return fail(LESBGK_EINVAL, "rows %d too short for ny %d", rows, sl.p.ny);
+  return 0;
+}
+
+}  // namespace
+
+extern "C" int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream) {
+  if (!b) return fail(LESBGK_EINVAL, "batch is NULL");
+  if (int rc = check_rows(b, rows)) return rc;
   b->rows = rows;
   b->auto_rows = false;
   drop_graph(b);
@@ -1796,83 +1807,102 @@ extern "C" int lesbgk_batch_get_work(lesbgk_batch *b, int32_t slot, int32_t *ste
   return 0;
 }
 
-extern "C" int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates, int32_t n, int32_t *chosen,
-                                     void *stream) {
-  lesbgk_internal::Range range_("lesbgk_batch_autotune");
-  if (!b || !candidates || n < 1) return fail(LESBGK_EINVAL, "bad autotune arguments");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaStream_t s2 = nullptr, sc[kChains - 1] = {};  // resident launches; chains past the first
-  cudaEvent_t t0, t1, fork, join;
+namespace {
+
+// How a batch's steps are launched, as the caller or the rules chose it.
+struct LaunchConfig {
+  bool auto_rows, auto_resident, resident;
+  int rows, resident_k, resident_limit;
+};
+
+LaunchConfig launch_config(const lesbgk_batch *b) {
+  return {b->auto_rows, b->auto_resident, b->resident, b->rows, b->resident_k, b->resident_limit};
+}
+
+void set_launch_config(lesbgk_batch *b, const LaunchConfig &c) {
+  b->auto_rows = c.auto_rows;
+  b->auto_resident = c.auto_resident;
+  b->resident = c.resident;
+  b->rows = c.rows;
+  b->resident_k = c.resident_k;
+  b->resident_limit = c.resident_limit;
+  drop_graph(b);
+  b->items_dirty = true;
+}
+
+const LaunchConfig kRules = {true, true, true, 32, 64, 128};  // as a batch is created
+
+// The fastest of the candidate rows x {per-step kernel for all, resident kernel
+// with 16 or 64 steps per launch for solves of at most so many rows} and, where
+// asked for, the rules.  Each is timed as the step graph it would run (launches
+// from the host took longer than the steps of small batches, and chose wrongly:
+// 64 short channels ended at 3.8 us per step, now 2.1).
+int tune(lesbgk_batch *b, const int32_t *candidates, int n, bool rules, int32_t *chosen, cudaStream_t s) {
+  const LaunchConfig entry = launch_config(b);
+  std::vector<LaunchConfig> cands;
+  if (rules) cands.push_back(kRules);
+  for (int c = 0; c < n; ++c) {
+    if (int rc = check_rows(b, candidates[c])) return rc;
+    cands.push_back({false, false, false, candidates[c], entry.resident_k, entry.resident_limit});
+    for (int lim : {64, 128, 256, 1 << 30})
+      for (int k : {16, 64}) cands.push_back({false, false, true, candidates[c], k, lim});
+  }
+  cudaEvent_t t0 = nullptr, t1 = nullptr;
   cudaError_t e = cudaEventCreate(&t0);
   if (e == cudaSuccess) e = cudaEventCreate(&t1);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s2, cudaStreamNonBlocking);
-  for (cudaStream_t &x : sc)
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking);
-  if (e != cudaSuccess) return cuda_fail(e, "autotune set-up");
-  // candidates: rows per work item x {per-step kernel for all, resident
-  // kernel with 16 or 64 steps per launch}; each timed as a 64-step chunk,
-  // the chains and the resident launches on streams beside one another (as in
-  // the graph), every launch reading the current buffers and writing the
-  // spare ones, so the state is left untouched
-  struct Cand { int rows, res, k, limit; };
-  std::vector<Cand> cands;
-  for (int c = 0; c < n; ++c) {
-    cands.push_back({candidates[c], 0, b->resident_k, b->resident_limit});
-    for (int lim : {64, 128, 256, 1 << 30})
-      for (int k : {16, 64}) cands.push_back({candidates[c], 1, k, lim});
-  }
-  b->auto_resident = false;
-  Cand best{b->rows, b->resident ? 1 : 0, b->resident_k, b->resident_limit};
+  LaunchConfig best = entry;
   float best_ms = 1e30f;
   int rc = 0;
-  for (const Cand &cd : cands) {
-    b->resident = cd.res != 0;
-    b->resident_k = cd.k;
-    b->resident_limit = cd.limit;
-    if ((rc = lesbgk_batch_set_rows(b, cd.rows, stream))) break;
+  for (const LaunchConfig &cd : cands) {
+    if (e != cudaSuccess) break;
+    set_launch_config(b, cd);
+    if ((rc = ensure_items(b, s)) || (rc = build_graph(b, true))) break;
     float ms = 0;
-    for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
+    auto chunks = [&](int count) {  // ms per chunk, back to back as lesbgk_batch_step runs them
       e = cudaEventRecord(t0, s);
-      if (e == cudaSuccess) e = cudaEventRecord(fork, s);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(s2, fork, 0);
-      for (cudaStream_t x : sc)
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(x, fork, 0);
-      for (int c = 0; c < kGraphSteps / cd.k && e == cudaSuccess; ++c) e = launch_resident(b, cd.k, b->par, b->par ^ 1, s2);
-      if (e == cudaSuccess) e = cudaEventRecord(join, s2);
-      for (int st = 0; st < kGraphSteps && e == cudaSuccess; ++st)
-        for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls)
-          for (int c = 0; c < kChains && e == cudaSuccess; ++c)
-            if (b->range_chain[cls][c][1]) e = launch_one_step(b, cls, b->par, c ? sc[c - 1] : s, c);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join, 0);
-      for (cudaStream_t x : sc) {
-        if (e == cudaSuccess) e = cudaEventRecord(join, x);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join, 0);
-      }
+      for (int k = 0; k < count && e == cudaSuccess; ++k) e = cudaGraphLaunch(b->graph, s);
       if (e == cudaSuccess) e = cudaEventRecord(t1, s);
       if (e == cudaSuccess) e = cudaEventSynchronize(t1);
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
-    }
-    if (e != cudaSuccess) break;
-    if (ms < best_ms) {
+      ms /= (float)count;
+    };
+    chunks(1);  // warms up; far behind the best, it decides
+    if (e == cudaSuccess && ms < 1.5f * best_ms) chunks(2);
+    if (e == cudaSuccess && ms < best_ms) {
       best_ms = ms;
       best = cd;
     }
   }
-  cudaEventDestroy(t0);
-  cudaEventDestroy(t1);
-  cudaEventDestroy(fork);
-  cudaEventDestroy(join);
-  cudaStreamDestroy(s2);
-  for (cudaStream_t x : sc) cudaStreamDestroy(x);
+  if (t0) cudaEventDestroy(t0);
+  if (t1) cudaEventDestroy(t1);
+  const bool failed = rc || e != cudaSuccess;
+  set_launch_config(b, failed ? entry : best);
   if (rc) return rc;
   if (e != cudaSuccess) return cuda_fail(e, "autotune");
-  b->resident = best.res != 0;
-  b->resident_k = best.k;
-  b->resident_limit = best.limit;
-  if (chosen) *chosen = best.rows;
-  return lesbgk_batch_set_rows(b, best.rows, stream);
+  if (chosen) *chosen = best.auto_rows ? 0 : best.rows;
+  return ensure_items(b, s);
+}
+
+}  // namespace
+
+extern "C" int lesbgk_batch_autotune(lesbgk_batch *b, const int32_t *candidates, int32_t n, int32_t *chosen,
+                                     void *stream) {
+  lesbgk_internal::Range range_("lesbgk_batch_autotune");
+  if (!b || !candidates || n < 1) return fail(LESBGK_EINVAL, "bad autotune arguments");
+  return tune(b, candidates, n, false, chosen, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" int lesbgk_batch_autotune_rules(lesbgk_batch *b, const int32_t *candidates, int32_t n, int32_t *chosen,
+                                           void *stream) {
+  lesbgk_internal::Range range_("lesbgk_batch_autotune");
+  if (!b || !candidates || n < 1) return fail(LESBGK_EINVAL, "bad autotune arguments");
+  return tune(b, candidates, n, true, chosen, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" int lesbgk_batch_set_auto(lesbgk_batch *b, void *stream) {
+  if (!b) return fail(LESBGK_EINVAL, "batch is NULL");
+  set_launch_config(b, kRules);
+  return ensure_items(b, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int lesbgk_batch_check_guards(lesbgk_batch *b, int32_t *h_bad, void *stream) {

@@ -37,7 +37,8 @@ SYMBOLS = ("lesbgk_workspace_size", "lesbgk_create", "lesbgk_reinit", "lesbgk_st
            "lesbgk_batch_autotune", "lesbgk_batch_pool_free", "lesbgk_batch_destroy", "lesbgk_batch_add_many",
            "lesbgk_batch_moments_many", "lesbgk_batch_set_resident", "lesbgk_batch_get_launch",
            "lesbgk_batch_check_guards", "lesbgk_batch_debug_poison", "lesbgk_batch_raw_bytes",
-           "lesbgk_batch_get_raw", "lesbgk_batch_set_raw", "lesbgk_on_chip_ctas", "lesbgk_batch_get_work")
+           "lesbgk_batch_get_raw", "lesbgk_batch_set_raw", "lesbgk_on_chip_ctas", "lesbgk_batch_get_work",
+           "lesbgk_batch_set_auto", "lesbgk_batch_autotune_rules")
 
 
 class Params(C.Structure):
@@ -119,6 +120,8 @@ def lib():
             L.lesbgk_batch_get_info.argtypes = [vp, i32, C.POINTER(Info)]
             L.lesbgk_batch_set_rows.argtypes = [vp, i32, vp]
             L.lesbgk_batch_autotune.argtypes = [vp, vp, i32, C.POINTER(i32), vp]
+            L.lesbgk_batch_autotune_rules.argtypes = [vp, vp, i32, C.POINTER(i32), vp]
+            L.lesbgk_batch_set_auto.argtypes = [vp, vp]
             L.lesbgk_batch_pool_free.argtypes = [vp, C.POINTER(sz), C.POINTER(sz)]
             L.lesbgk_batch_check_guards.argtypes = [vp, vp, vp]
             L.lesbgk_batch_raw_bytes.argtypes = [vp, i32, C.POINTER(sz)]
@@ -464,12 +467,19 @@ class Batch:
     def set_rows(self, rows: int) -> None:
         _check(lib().lesbgk_batch_set_rows(C.c_void_p(self.handle), C.c_int32(rows), self._s))
 
-    def autotune(self, candidates=(8, 16, 32, 64, 128)) -> int:
-        arr = (C.c_int32 * len(candidates))(*candidates)
+    def autotune(self, candidates=None) -> int:
+        """Keep the fastest launch configuration and return its rows per item: among the caller's
+        candidate rows, or, without any, among 8 to 128 rows and the batch's own rules."""
+        rows = (8, 16, 32, 64, 128) if candidates is None else candidates
+        arr = (C.c_int32 * len(rows))(*rows)
         chosen = C.c_int32()
-        _check(lib().lesbgk_batch_autotune(C.c_void_p(self.handle), arr, C.c_int32(len(candidates)),
-                                           C.byref(chosen), self._s))
-        return chosen.value
+        call = lib().lesbgk_batch_autotune_rules if candidates is None else lib().lesbgk_batch_autotune
+        _check(call(C.c_void_p(self.handle), arr, C.c_int32(len(rows)), C.byref(chosen), self._s))
+        return chosen.value or self.launch()["rows_per_item"]
+
+    def set_auto(self) -> None:
+        """Rows, chains and the resident kernel by the batch's contents, as it was created."""
+        _check(lib().lesbgk_batch_set_auto(C.c_void_p(self.handle), self._s))
 
     def set_resident(self, on: bool, steps_per_launch: int = 0, max_ny: int = 0) -> None:
         _check(lib().lesbgk_batch_set_resident(C.c_void_p(self.handle), C.c_int32(1 if on else 0),

@@ -498,3 +498,40 @@ def test_large_and_pinned_fields_arrive_whole(capacity, sizes, pinned):
         assert int(many.check_guards().sum()) == 0
         for s in slots:
             many.remove(s)
+
+
+def test_autotune_may_keep_the_rules_and_a_failed_one_changes_nothing():
+    """Without candidates of the caller's the tuner keeps the batch's own rules
+    where they win (they do against rows no solve here should run with), with
+    the state untouched; a call that fails leaves the configuration as it was;
+    set_auto returns to the rules."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    probs = I.batch_mix(n=150, seed=150, ny_lo=600, ny_hi=1024)
+    bt, params, slots = _batch(probs)
+    ref, _, slots2 = _batch(probs)
+    bt.step(3)  # an odd parity
+    rules = bt.work(slots[0]), bt.launch()
+    before = [bt.populations(s) for s in slots]
+    assert bt.autotune() == rules[1]["rows_per_item"]
+    assert (bt.work(slots[0]), bt.launch()) == rules
+    assert all(torch.equal(bt.populations(s), x) for s, x in zip(slots, before))
+    for rows in ((64, 0), (64, 5000), (64, -1)):
+        with pytest.raises(L.LesbgkError) as err:
+            bt.autotune(rows)
+        assert err.value.code == L.EINVAL and (bt.work(slots[0]), bt.launch()) == rules
+    assert bt.autotune((64, 128)) in (64, 128)
+    fixed = bt.work(slots[0]), bt.launch()
+    assert fixed[0]["step_rows"] in (0, 64, 128) and fixed[1] != rules[1]
+    with pytest.raises(L.LesbgkError):
+        bt.autotune((32, 4097))
+    assert (bt.work(slots[0]), bt.launch()) == fixed
+    bt.set_auto()
+    assert (bt.work(slots[0]), bt.launch()) == rules
+    bt.step(64 + 6)
+    ref.step(73)
+    for s, t in zip(slots, slots2):
+        assert torch.equal(bt.populations(s), ref.populations(t))
+    empty = L.Batch(capacity=2, nx=4, pool_bytes=1 << 20)
+    assert empty.autotune((8, 16)) in (8, 16)
