@@ -438,8 +438,6 @@ def measure_batch_fixed(params, nsteps, passes, warmup, stream, local, plain_sam
             bt.remove(s)
         return bt.add_many(params)  # one descriptor copy, one init launch
 
-    admit_all()
-    rows = bt.autotune((2, 4, 8, 16, 32, 64))
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")  # larger than the 129 MB L2
 
     def one_pass():
@@ -451,24 +449,26 @@ def measure_batch_fixed(params, nsteps, passes, warmup, stream, local, plain_sam
     for _ in range(warmup):
         one_pass()
     torch.cuda.synchronize()
-    launch = bt.launch()  # the autotuner's choice
+    launch = bt.launch()  # the rules' choice for these solves
+    rows = launch["rows_per_item"]
 
     def time_steps():
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         admit_all()
+        bt.step(64)  # builds the step graph of this mode
         e0.record(stream)
         bt.step(640)
         e1.record(stream)
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / 640
 
-    # one batch step of all instances, per launch mode (the chosen one last)
+    # one batch step of all instances, per launch mode (the rules last)
     modes = {}
     for name, on, k, lim in (("per_step_only", False, 64, 128), ("resident_k64_ny64", True, 64, 64),
                              ("resident_k64_ny128", True, 64, 128), ("resident_k64_all", True, 64, 1 << 20)):
         bt.set_resident(on, k, lim)
         modes[name] = time_steps()
-    bt.set_resident(launch["resident"], launch["steps_per_launch"], launch["resident_max_ny"])
+    bt.set_auto()
     step_ms = time_steps()
     with ClockSampler(local) as clk:
         barrier()
