@@ -43,6 +43,11 @@ constexpr int kBRing = 4;
 constexpr int kNumClasses = 18;
 constexpr int kGraphSteps = 64;
 constexpr int kChains = 4;  // at most: independent chains of steps a class's solves are dealt to
+// ... and about this many over all classes, which step side by side anyway: with
+// four each, 18 classes of 662 solves (32 columns) took 227 us per step, at 24,
+// 16, 12, 8, 6 chains in all 154; six classes of 2000 channels 171 us, at 16 152,
+// at 8 and 6 137; three of them 108 and 105, two the same
+constexpr int kChainsInAll = 8;
 constexpr size_t kGuardBytes = 256;       // guard words after each slot's pool block
 constexpr unsigned char kGuardByte = 0xA5;
 // a batch whose solves all have at most this many rows goes to the resident
@@ -971,7 +976,7 @@ cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s, i
 
 // Rows per work item and chains of each class, from the solves it holds, until
 // the caller sets rows: items for one and a half times the blocks its share of
-// the chip holds (by work: the classes run side by side), dealt to kChains
+// the chip holds (by work: the classes run side by side), dealt to up to kChains
 // chains once they fill it.  A step's launch, first loads and last blocks cost
 // about 4 us whatever its size; beside three other chains that time is filled
 // (512 channels of 16 to 1024 rows, us per step with one chain at its best
@@ -987,7 +992,12 @@ void pick_rows(lesbgk_batch *b) {
     rows[sl.cls] += sl.p.ny;
     work[sl.cls] += (double)sl.p.ny * stored_values(sl.p);
   }
-  for (double w : work) all += w;
+  int active = 0;  // classes with steps
+  for (double w : work) {
+    all += w;
+    active += w > 0.0;
+  }
+  const int most = std::max(1, std::min(kChains, kChainsInAll / std::max(active, 1)));
   const double sms = b->sm_count > 0 ? b->sm_count : 152;
   const double per_block = (double)(kBBlock / b->W);  // items a block takes
   for (int cls = 0; cls < kNumClasses; ++cls) {
@@ -1001,7 +1011,7 @@ void pick_rows(lesbgk_batch *b) {
     const double cap = (cls % 3 == 0 ? 4 : 2) * sms * work[cls] / all;
     int r = b->rows;
     if (b->auto_rows) r = (int)std::fmin(64.0, std::ceil(rows[cls] / (per_block * 1.5 * cap)));
-    auto chains = [&](int at) { return rows[cls] / (per_block * at) > 0.75 * cap ? kChains : 1; };
+    auto chains = [&](int at) { return rows[cls] / (per_block * at) > 0.75 * cap ? most : 1; };
     const int old = b->rows_of[cls];
     if (b->auto_rows && b->graph && old && 2 * old >= r && old <= 2 * r && b->chains_of[cls] == chains(old) &&
         rows[cls] / (per_block * old) / b->chains_of[cls] + 1.0 < b->graph_grid[cls][0])

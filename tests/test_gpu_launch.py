@@ -535,3 +535,26 @@ def test_autotune_may_keep_the_rules_and_a_failed_one_changes_nothing():
         assert torch.equal(bt.populations(s), ref.populations(t))
     empty = L.Batch(capacity=2, nx=4, pool_bytes=1 << 20)
     assert empty.autotune((8, 16)) in (8, 16)
+
+
+@pytest.mark.parametrize("classes,chains", [(1, 4), (2, 4), (3, 2), (6, 1)])
+def test_chains_are_shared_among_the_classes(classes, chains):
+    """However many classes a batch holds, about eight chains step it, with the
+    bits of fixed rows."""
+    import torch
+    from dataclasses import replace
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    kinds = [(4, 2, 0), (6, 2, 0), (4, 3, 0), (4, 2, 1), (6, 2, 1), (4, 3, 2)][:classes]
+    probs = [replace(p, nroots=kinds[k % classes][0], dim=kinds[k % classes][1])
+             for k, p in enumerate(I.batch_mix(n=192, seed=9, ny_lo=200, ny_hi=1024))]
+    got = []
+    for kw in ({}, {"set_resident": False, "set_rows": 32}):
+        bt, params, slots = _batch(probs, storage=[k[2] for k in kinds], **kw)
+        if not kw:
+            assert {bt.work(s)["chains"] for s in slots} == {chains}
+        bt.step(64 + 1)
+        got.append([bt.populations(s) for s in slots])
+        bt.close()
+    for a, b in zip(*got):
+        assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
