@@ -370,8 +370,8 @@ int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream);
  * 64-step graphs the two run side by side.  A resident instance is one
  * block's serial work, so tall ones are better left to the per-step kernel:
  * until this call (or lesbgk_batch_autotune), and again from
- * lesbgk_batch_set_auto, it is on where every solve of the batch has at most 64
- * rows, and off otherwise.
+ * lesbgk_batch_set_auto, it is on where every solve of the batch is such an
+ * instance of at most 256 nodes, and off otherwise.
  * Results do not depend on the choice (bitwise). */
 int lesbgk_batch_set_resident(lesbgk_batch *b, int32_t on, int32_t steps_per_launch, int32_t max_ny, void *stream);
 /* The launch configuration in use (any pointer may be NULL). */

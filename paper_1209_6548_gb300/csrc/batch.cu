@@ -50,12 +50,14 @@ constexpr int kChains = 4;  // at most: independent chains of steps a class's so
 constexpr int kChainsInAll = 8;
 constexpr size_t kGuardBytes = 256;       // guard words after each slot's pool block
 constexpr unsigned char kGuardByte = 0xA5;
-// a batch whose solves all have at most this many rows goes to the resident
-// kernel by default (64 channels, us per step, per-step kernel against
-// resident: up to 32 rows 2.8 and 1.1, up to 64 rows 2.9 and 2.1, up to 128
-// rows 3.1 and 3.7); beside taller ones, whose steps set the pace, it only
-// takes their slots (256 channels up to 512 rows: 6.5 and 6.7)
-constexpr int kAutoResidentNy = 64;
+// A batch whose solves all have at most this many nodes (two per thread), and
+// rows within the resident kernel's limit, goes to it by default: us per step of
+// 64 solves, per-step kernel against resident: 64 rows of 1, 2, 4 columns 3.0 and
+// 1.2, 2.8 and 1.3, 2.9 and 2.1; 128 rows 3.0 and 1.2, 2.8 and 2.3, 2.8 and 3.7;
+// 8 columns of 32 and 64 rows 2.8 and 2.1, 2.8 and 3.7; 32 of 8 and 16 rows 2.6
+// and 2.1, 2.5 and 3.7.  Beside taller ones, whose steps set the pace, it only
+// takes their slots (256 channels up to 512 rows: 6.5 and 6.7).
+constexpr int kAutoResidentNodes = 256;
 constexpr int kBuckets = 6;  // resident instances by height: ny <= 16, 32, ..., 512 (smem permitting)
 
 // Per-instance descriptor (device memory).
@@ -1030,7 +1032,7 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
   if (b->auto_resident) {
     b->resident = true;
     for (const auto &sl : b->slots)
-      if (sl.used && (sl.cls != 0 || sl.p.ny > std::min(b->resident_ny, kAutoResidentNy))) b->resident = false;
+      if (sl.used && (!is_resident(b, sl) || sl.p.nx * sl.p.ny > kAutoResidentNodes)) b->resident = false;
   }
   pick_rows(b);
   // Residuals and moments read every solve in items of their own, of the

@@ -558,3 +558,23 @@ def test_chains_are_shared_among_the_classes(classes, chains):
         bt.close()
     for a, b in zip(*got):
         assert bool(torch.isfinite(a).all()) and torch.equal(a, b)
+
+
+@pytest.mark.parametrize("nx,ny,resident", [(1, 128, True), (1, 129, False), (2, 128, True), (2, 129, False), (4, 64, True),
+                                            (4, 65, False), (8, 32, True), (8, 33, False), (32, 8, True), (32, 9, False)])
+def test_which_batches_are_resident(nx, ny, resident):
+    """Solves of at most 256 nodes and 128 rows go to the resident kernel by
+    themselves, with the bits of the per-step kernel; one that does not keeps
+    all of them from it."""
+    import torch
+    from dataclasses import replace
+
+    probs = [replace(I.batch_mix(n=1, seed=1)[0], nx=nx, ny=h) for h in (ny, max(4, ny // 2), 4)]
+    bt, _, slots = _batch(probs)
+    ref, _, slots2 = _batch(probs, set_resident=False)
+    for s in slots:
+        assert (bt.work(s)["step_rows"] == 0) == resident
+    for x in (bt, ref):
+        x.step(64 + 3)
+    for s, t in zip(slots, slots2):
+        assert torch.equal(bt.populations(s), ref.populations(t))
