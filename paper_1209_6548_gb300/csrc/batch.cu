@@ -152,14 +152,17 @@ __device__ __forceinline__ void wall_fix_heated(float (&O)[Q], int side, const T
 // One time step of every work item of a class (velocity set and storage S:
 // FP32 deviations, or FP16/BF16 relative deviations rounded stochastically
 // with the random words of k_step, keyed by the instance's step count and row).
-// What bounds it: issue (D2Q16: 740 instructions per node and step in short items,
-// 600 in long ones: 553k nodes cannot take less than 8.5 us on 152 SMs) and the latency of each warp's
-// chain, so it needs warps: the per-item coefficients and flags sit in shared
-// memory (a dozen 16-byte reads per row) instead of registers, which lets
-// D2Q16 keep four blocks on an SM (165 -> 128 registers) and D2Q36 run
-// without spills (96 B before), on packed pairs.
-template <int NR, int N, int W, class S, bool HEAT, int NZ>
-__global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_step(const BatchArgs B, const int par) {
+// What bounds it: issue (D2Q16: 740 instructions per node and step in items of six
+// rows, 600 in long ones: at 2070 MHz 553k nodes cannot take less than 10.2 and
+// 8.2 us on 152 SMs) and the latency of each warp's chain, so it needs warps: the
+// per-item coefficients and flags sit in shared memory (a dozen 16-byte reads per
+// row) instead of registers, which lets D2Q16 keep four blocks on an SM (165 ->
+// 128 registers) and D2Q36 run without spills (96 B before), on packed pairs.
+// FEW: for steps that leave the chip part full (StepChoice), D2Q16 on three
+// blocks with the flags in registers.
+template <int NR, int N, int W, class S, bool HEAT, int NZ, bool FEW>
+__global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? (FEW ? 3 : 4) : 2)
+    k_batch_step(const BatchArgs B, const int par) {
   using Lay = Layout<NR, S, NZ>;
   constexpr int Q = Lay::Q, H = Lay::H, V = Lay::V, G = Lay::G;
   constexpr int GPW = 32 / W;
@@ -179,7 +182,7 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
   // this group's coefficients: entry c at coef[c * GPW], one broadcast per group
   float4 *coef = reinterpret_cast<float4 *>(smem_raw + kBatchRingBytes<NR, S, NZ>) +
                  (threadIdx.x >> 5) * kCoefs<NR> * GPW + gi;
-  for (int c = lx; c < kCoefs<NR>; c += W) {
+  auto entry = [&](int c) {
     float4 v;
     if (c < NR) {
       v = make_float4(D.kx[c], D.kx[c], -D.ax[c], -D.ax[c]);
@@ -197,9 +200,22 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
       v = make_float4(__int_as_float((int)(unsigned)o), __int_as_float((int)(unsigned)(o >> 32)),
                       __int_as_float(live ? wi.rows : 0), __int_as_float(wi.y0));
     }
-    coef[c * GPW] = v;
+    return v;
+  };
+  // From four lanes a group on, a lane's few entries wait in registers until the
+  // first rows are on their way, so that an item waits for memory once (us per
+  // step: 512 channels 12.6 -> 12.3, D3Q64 28.4 -> 27.6, 96 of D2Q36 6.5 -> 5.9).
+  constexpr bool kHold = W >= 4;
+  constexpr int kMine = (kCoefs<NR> + W - 1) / W;
+  [[maybe_unused]] float4 held[kHold ? kMine : 1];
+  if constexpr (kHold) {
+#pragma unroll
+    for (int i = 0; i < kMine; ++i)
+      if (lx + i * W < kCoefs<NR>) held[i] = entry(lx + i * W);
+  } else {
+    for (int c = lx; c < kCoefs<NR>; c += W) coef[c * GPW] = entry(c);
+    __syncwarp();
   }
-  __syncwarp();
   const S *fin = reinterpret_cast<const S *>(D.f[par]);
   const long long gstride = (long long)V * W * ny;
   const long long rstride = (long long)V * W;
@@ -225,6 +241,12 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
       if (g >= G / 2) ld_group_cg<NR, S>(pm2, gstride, g, m2, B.lat);
       else ld_group_cg<NR, S>(pp1, gstride, g, p1, B.lat);
     }
+    if constexpr (kHold) {
+#pragma unroll
+      for (int i = 0; i < kMine; ++i)
+        if (lx + i * W < kCoefs<NR>) coef[(lx + i * W) * GPW] = held[i];
+      __syncwarp();
+    }
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
       if (a % NR >= H) {
@@ -242,9 +264,18 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
   int r1 = map_row(y0 + 1, ny, walls), r2 = map_row(y0 + 2, ny, walls);
   const int4 *iflags = reinterpret_cast<const int4 *>(coef + (kCoefScalars<NR> + 2) * GPW);
   const int4 *iout = reinterpret_cast<const int4 *>(coef + (kCoefScalars<NR> + 3) * GPW);
+  [[maybe_unused]] int4 fl_few, out_few;
+  if constexpr (FEW) {
+    fl_few = *iflags;
+    out_few = *iout;
+  }
+  auto flags = [&] {
+    if constexpr (FEW) return fl_few;
+    else return *iflags;
+  };
   auto issue_rowload = [&](int k) {
     if (k < nrows) {
-      const int2 fl = *reinterpret_cast<const int2 *>(iflags);  // ny, walls
+      const int4 fl = flags();
       const long long gstride = (long long)(V * W) * fl.x;
       const S *q1 = fx + r1 * rstride, *q2 = fx + r2 * rstride;
       T *slot = ring + (k % kBRing) * G * 32;
@@ -277,7 +308,7 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
     float xs[Q];
     const GroupLanes nb{srcL, srcR};
     const float2 omw2 = make_float2(omw, omw);
-    const int4 fl = *iflags;
+    const int4 fl = flags();
     // the printed update's x-fluxes take f^n itself: a selection, since a zero
     // coefficient would turn an infinite y-flux into NaN (0 Inf) there (it was
     // that, 512 channels: D2Q16 13.3 us per step, now 13.5, D2Q36 41.7 -> 42.4,
@@ -321,7 +352,9 @@ __global__ void __launch_bounds__(kBBlock, NZ * NR * NR == 16 ? 4 : 2) k_batch_s
           acc[a + 1] = ac.y;
         }
     }
-    const int4 out = *iout;
+    int4 out;
+    if constexpr (FEW) out = out_few;
+    else out = *iout;
     const int j = out.w + k;
     if (fl.y && (j == 0 || j == fl.x - 1)) {
       const int side = j == 0 ? 0 : 1;
@@ -736,6 +769,24 @@ void with_class(int cls, Fn &&fn) {
 
 }  // namespace
 
+// How a class's steps are launched beside its rows and chains.
+//   few: D2Q16 that leaves the chip part full takes the three-block kernel, whose
+//     rows are shorter chains (512 channels at the caller's 32 rows 23.4 us per
+//     step on the four-block kernel, 21.9 on it).  By default rows, four-block
+//     kernel against it: 4 columns, 300 blocks 4.24 and 4.15, 400 in one chain
+//     4.40 and 5.02, 460 in four 5.08 and 4.64, 640 5.5 and 4.9, 1200 the same;
+//     16 columns, 400 blocks 4.31 and 3.86, 520 4.12 and 4.18, 640 4.3 and 5.1.
+//     Beside other classes only with rows of the caller's.
+//   drain: with the caller's rows, a lone chain of long items that leaves SMs
+//     part full starts each step after the previous one's end; blocks that
+//     enter as others leave would crowd (512 channels of 16 and 32 rows 23.2 and
+//     26.2 against 18.0 and 21.9 drained; D3Q64 of 32 rows 49.9 and 41.9).  Below
+//     0.55 blocks per SM, above two, or with fewer than 8 rows (4 on the wide
+//     sets) overlapping is the faster one (32 rows of 96 channels 21.2 and 21.6).
+struct StepChoice {
+  bool few, drain;
+};
+
 struct lesbgk_batch {
   struct Slot {
     bool used = false;
@@ -782,6 +833,7 @@ struct lesbgk_batch {
   int rows = 32;           // rows per work item where the caller sets them
   bool auto_rows = true;   // until then: rows and chains per class by pick_rows
   int rows_of[kNumClasses] = {}, chains_of[kNumClasses] = {};
+  StepChoice choice_of[kNumClasses] = {};
   int par = 0;
   int sm_count = 0;
   LatTables lat[kNumClasses];
@@ -860,22 +912,33 @@ char *guard_of(const lesbgk_batch *b, const lesbgk_batch::Slot &sl) {
 
 bool pow2_le32(int n) { return n >= 1 && n <= 32 && (n & (n - 1)) == 0; }
 
-template <int NR, int N, class S, bool HEAT, int NZ>
+template <int NR, int N, class S, bool HEAT, int NZ, bool FEW>
 void *step_fn(int W) {
   switch (W) {
-    case 1: return (void *)k_batch_step<NR, N, 1, S, HEAT, NZ>;
-    case 2: return (void *)k_batch_step<NR, N, 2, S, HEAT, NZ>;
-    case 4: return (void *)k_batch_step<NR, N, 4, S, HEAT, NZ>;
-    case 8: return (void *)k_batch_step<NR, N, 8, S, HEAT, NZ>;
-    case 16: return (void *)k_batch_step<NR, N, 16, S, HEAT, NZ>;
-    default: return (void *)k_batch_step<NR, N, 32, S, HEAT, NZ>;
+    case 1: return (void *)k_batch_step<NR, N, 1, S, HEAT, NZ, FEW>;
+    case 2: return (void *)k_batch_step<NR, N, 2, S, HEAT, NZ, FEW>;
+    case 4: return (void *)k_batch_step<NR, N, 4, S, HEAT, NZ, FEW>;
+    case 8: return (void *)k_batch_step<NR, N, 8, S, HEAT, NZ, FEW>;
+    case 16: return (void *)k_batch_step<NR, N, 16, S, HEAT, NZ, FEW>;
+    default: return (void *)k_batch_step<NR, N, 32, S, HEAT, NZ, FEW>;
   }
 }
 
-void *step_kernel(int cls, int W) {
+bool few_built(int cls) { return cls % 3 == 0; }  // D2Q16, whatever its storage and heating
+
+void *step_kernel(int cls, int W, bool few) {
   void *fn = nullptr;
   with_class(cls, [&](auto r, auto n, auto st, auto ht, auto z) {
-    fn = step_fn<decltype(r)::value, decltype(n)::value, decltype(st), decltype(ht)::value, decltype(z)::value>(W);
+    constexpr int NR = decltype(r)::value, N = decltype(n)::value, NZ = decltype(z)::value;
+    using S = decltype(st);
+    constexpr bool HEAT = decltype(ht)::value;
+    if constexpr (NZ * NR * NR == 16) {
+      if (few) {
+        fn = step_fn<NR, N, S, HEAT, NZ, true>(W);
+        return;
+      }
+    }
+    fn = step_fn<NR, N, S, HEAT, NZ, false>(W);
   });
   return fn;
 }
@@ -957,15 +1020,14 @@ unsigned step_grid(const lesbgk_batch *b, int n_items) {
   return (unsigned)std::max<long long>(blocks, 1);
 }
 
-// One step of a class, or of one of its chains.
-cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s, int chain = -1) {
+// One step of a class.
+cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s) {
   BatchArgs a = make_args(b, cls);
-  if (chain >= 0) a.range = chain_range(b, cls, chain);
-  const unsigned grid = step_grid(b, chain < 0 ? b->range[cls][1] : b->range_chain[cls][chain][1]);
+  const unsigned grid = step_grid(b, b->range[cls][1]);
   void *args[] = {&a, &par};
   cudaLaunchAttribute at{};  // may be scheduled while the previous step runs (the kernel waits for it)
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+  at.val.programmaticStreamSerializationAllowed = b->choice_of[cls].drain ? 0 : 1;
   cudaLaunchConfig_t c{};
   c.gridDim = dim3(grid);
   c.blockDim = dim3(kBBlock);
@@ -973,7 +1035,7 @@ cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s, i
   c.stream = s;
   c.attrs = &at;
   c.numAttrs = 1;
-  return cudaLaunchKernelExC(&c, step_kernel(cls, b->W), args);
+  return cudaLaunchKernelExC(&c, step_kernel(cls, b->W, b->choice_of[cls].few), args);
 }
 
 // Rows per work item and chains of each class, from the solves it holds, until
@@ -1020,6 +1082,14 @@ void pick_rows(lesbgk_batch *b) {
       continue;
     b->rows_of[cls] = r;
     b->chains_of[cls] = chains(r);
+    const double blocks = rows[cls] / (per_block * r);
+    StepChoice &c = b->choice_of[cls];
+    const bool d2q16 = few_built(cls);
+    c.few = d2q16 && (active == 1 || !b->auto_rows) &&
+            (b->W > 4 ? blocks < 0.8 * cap
+                      : blocks < 0.5 * cap || (b->chains_of[cls] > 1 && blocks < 1.1 * cap));
+    c.drain = !b->auto_rows && b->chains_of[cls] == 1 && r >= (d2q16 ? 8 : 4) && blocks > 0.55 * sms &&
+              blocks <= 2.0 * sms;
   }
 }
 
@@ -1161,14 +1231,15 @@ int build_graph(lesbgk_batch *b, bool timing = false) {
       if (!b->graph_grid[cls][c]) continue;
       cudaKernelNodeParams kp{};
       void *kargs[] = {&args[cls][c], &pars[st & 1]};
-      kp.func = step_kernel(cls, b->W);
+      kp.func = step_kernel(cls, b->W, b->choice_of[cls].few);
       kp.gridDim = dim3(b->graph_grid[cls][c]);
       kp.blockDim = dim3(kBBlock);
       kp.sharedMemBytes = (unsigned)step_smem(cls, b->W);
       kp.kernelParams = kargs;
       cudaGraphNode_t node;
       e = cudaGraphAddKernelNode(&node, g, nullptr, 0, &kp);
-      if (e == cudaSuccess && st) e = cudaGraphAddDependencies(g, &prev[cls][c], &node, &edge, 1);
+      if (e == cudaSuccess && st)
+        e = cudaGraphAddDependencies(g, &prev[cls][c], &node, b->choice_of[cls].drain ? nullptr : &edge, 1);
       prev[cls][c] = node;
     }
   }
@@ -1262,7 +1333,10 @@ extern "C" int lesbgk_batch_create(int32_t capacity, int32_t nx, void *d_workspa
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sm_count, cudaDevAttrMultiProcessorCount, dev);
   for (int w : {1, 2, 4, 8, 16, 32})
     for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls)
-      e = cudaFuncSetAttribute(step_kernel(cls, w), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem(cls, w));
+      for (bool few : {false, true})
+        if (e == cudaSuccess && (!few || few_built(cls)))
+          e = cudaFuncSetAttribute(step_kernel(cls, w, few), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)step_smem(cls, w));
   // the resident kernel: as tall an instance as two buffers of Q planes fit in
   // the opt-in shared memory of a block
   int optin = 0;

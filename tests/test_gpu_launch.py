@@ -578,3 +578,31 @@ def test_which_batches_are_resident(nx, ny, resident):
         x.step(64 + 3)
     for s, t in zip(slots, slots2):
         assert torch.equal(bt.populations(s), ref.populations(t))
+
+
+@pytest.mark.parametrize("nx,n,ny_hi", [(1, 70, 300), (2, 40, 200), (4, 60, 500), (8, 30, 200), (16, 24, 150), (32, 20, 120)])
+@pytest.mark.parametrize("nroots,dim,storage,amp", [(4, 2, 0, 0.0), (4, 2, 1, 0.0), (4, 2, 0, 0.02), (4, 2, 2, 0.02),
+                                                    (6, 2, 0, 0.0), (4, 3, 1, 0.0)])
+def test_any_rows_of_the_callers_give_the_bits_of_the_solve_alone(nx, n, ny_hi, nroots, dim, storage, amp):
+    """Rows from one to more than a solve has, which choose kernels, chains and
+    how steps follow one another: through graphs and single steps, every slot
+    as its solve alone, value for value and, where a solve diverges (some of the
+    shortest do), NaN for NaN."""
+    import torch
+    from dataclasses import replace
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    probs = [replace(p, nx=nx, nroots=nroots, dim=dim, scheme=I.SPLIT if k % 3 == 0 else I.UNSPLIT, wall_T_amp=amp,
+                     wall_T_freq=0.5 if amp else 0.0)
+             for k, p in enumerate(I.batch_mix(n=n, seed=n, ny_lo=3, ny_hi=ny_hi))]
+    bt, params, slots = _batch(probs, storage=(storage,), set_resident=False)
+    done = 0
+    for rows in (1, 2, 7, 16, 32, 64, 600):
+        bt.set_rows(rows)
+        bt.step(64 + 2)
+        done += 66
+    for k in range(0, n, 7):
+        ref = L.Solver(params[k])
+        ref.step(done)
+        got, want = bt.populations(slots[k]), ref.populations()
+        assert bool(((got == want) | (torch.isnan(got) & torch.isnan(want))).all()), (k, params[k].ny)
