@@ -1405,14 +1405,18 @@ int pick_launch(lesbgk *h) {
   // the ring's first loads, about kPro rows' time); a row takes one warp's
   // latency or, with k blocks on the SM, `base` + k times a block's `share` of
   // the issue slots, whichever is more (one-block against full-chip runs, in
-  // units of that latency); past one wave the blocks' ends are spread over half
-  // a segment.  Small grids so get short segments, middle ones the longest that
-  // fill every SM evenly (us per step with 32 or, D2Q36 and D3Q216, 128 rows ->
-  // now; 4x64 D2Q16 18.6 -> 2.7, D2Q36 70 -> 4.2; 256^2 cavity 25.6 -> 4.9;
-  // 512x1024 D2Q16 19.8 -> 14.3; 512^2 D2Q36 140 -> 18.0, D3Q64 33.0 -> 15.5).
-  // From two waves of `large` rows on, `large` is taken: 16 to 128 rows are
-  // within 4% there (4096^2 D2Q16: 367, 354, 361, 365 us at 16, 32, 64, 128;
-  // D3Q64: 808, 775, 777, 770).
+  // units of that latency).  Segments left over from a full wave share the slots
+  // it leaves free, and a last, partly filled wave runs at its own rate; short
+  // segments cost the wide sets one row more there (2500^2 D2Q36, 16 to 200 rows:
+  // within 1% of 1.035 times the model).  Small grids so get short segments,
+  // middle ones the longest that fill every SM evenly (us per step with 32 or,
+  // D2Q36 and D3Q216, 128 rows -> now; 4x64 D2Q16 18.6 -> 2.7, D2Q36 70 -> 4.2;
+  // 256^2 cavity 25.6 -> 4.9; 512x1024 D2Q16 19.8 -> 14.3; 512^2 D2Q36 140 -> 18.0,
+  // D3Q64 33.0 -> 15.5).  On 260 grids of every set and storage the choice is no
+  // slower than the fixed segments (D2Q36 6741x1242: 128 rows 458 us, 125 446; with
+  // waves counted as blocks / cap + 1/2 it was 27 rows, 493).  From two waves of
+  // `large` rows on, `large` is taken: 16 to 128 rows are within 4% there (4096^2
+  // D2Q16: 367, 354, 361, 365 us at 16, 32, 64, 128; D3Q64: 808, 775, 777, 770).
   constexpr double kPro = 1.5;
   const bool comp = h->p.storage == LESBGK_F32C, wide = h->q >= 32;
   const double slots = wide ? 2 : comp ? 3 : 4;  // blocks an SM holds (registers)
@@ -1437,9 +1441,18 @@ int pick_launch(lesbgk *h) {
         // SM gets a full set (1024^2 compensated: two of three slots, 32 rows,
         // 56 us per step; three of three, 21 rows, 40 us)
         if (2.0 * k > slots) k = slots;
-        if (blocks <= cap) t = (r + kPro) * std::fmax(1.0, base + share * k);
-        else if (whole <= cap) t = (r + kPro) * full + rest + kPro;  // the short segments follow the full wave
-        else t = full * (r + kPro) * (blocks / cap + 0.5);
+        if (blocks <= cap) {
+          t = (r + kPro) * std::fmax(1.0, base + share * k);
+        } else if (whole <= cap) {  // the short segments follow the full wave, or go through the slots it leaves
+          const double wave = (r + kPro) * full, free = cap - whole;
+          t = wave + rest + kPro;
+          if (free > 0.0)
+            t = std::fmin(t, std::fmax(wave, 1.05 * std::ceil((blocks - whole) / free) * (rest + kPro) * full));
+        } else {
+          const double waves = std::floor(blocks / cap), left = blocks - waves * cap;
+          const double last = left > 0.0 ? std::fmax(1.0, base + share * std::ceil(left / sms)) : 0.0;
+          t = (r + kPro + (wide && !comp ? 1.0 : 0.0)) * (waves * full + last);
+        }
         if (r == 1 || t <= best) {
           best = t;
           h->rows = r;

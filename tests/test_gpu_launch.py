@@ -606,3 +606,25 @@ def test_any_rows_of_the_callers_give_the_bits_of_the_solve_alone(nx, n, ny_hi, 
         ref.step(done)
         got, want = bt.populations(slots[k]), ref.populations()
         assert bool(((got == want) | (torch.isnan(got) & torch.isnan(want))).all()), (k, params[k].ny)
+
+
+@pytest.mark.parametrize("nroots,dim,nx,ny", [(6, 2, 2524, 1703), (6, 3, 2048, 1024), (4, 3, 2433, 1730)])
+def test_grids_just_past_a_wave_keep_long_segments(nroots, dim, nx, ny):
+    """Grids whose long segments take little more than whole waves keep them
+    (many short ones took 1 to 14% longer), with the bits of other rows."""
+    import torch
+    from paper_1209_6548_gb300 import lesbgk as L
+
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the waves are those of 152 SMs")
+    prob = I.Problem(name="wave", nroots=nroots, dim=dim, nx=nx, ny=ny, bc_y=I.PERIODIC, kn=0.1, b=-0.5, scheme=I.SPLIT)
+    p = L.params_from_problem(prob)
+    s = L.Solver(p, h_init=I.random_fields(prob, seed=1))
+    assert s.info.rows_per_segment >= 64
+    start = s.populations()
+    s.step(2)
+    got = s.populations()
+    s.set_populations(start, 0)
+    s.set_launch(0, 32)
+    s.step(2)
+    assert torch.equal(s.populations(), got)
