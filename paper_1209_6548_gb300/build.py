@@ -2,8 +2,8 @@
 
     python -m paper_1209_6548_gb300.build
 
-compiles csrc/lesbgk.cu and csrc/tables.cpp into
-paper_1209_6548_gb300/_build/liblesbgk.so.  The two translation units are
+compiles csrc/lesbgk.cu, batch.cu, setup.cpp and tables.cpp into
+paper_1209_6548_gb300/_build/liblesbgk.so.  The four translation units are
 compiled in parallel and linked with ``nvcc -shared``.
 """
 from __future__ import annotations

@@ -152,9 +152,9 @@ __device__ __forceinline__ void wall_fix_heated(float (&O)[Q], int side, const T
 // One time step of every work item of a class (velocity set and storage S:
 // FP32 deviations, or FP16/BF16 relative deviations rounded stochastically
 // with the random words of k_step, keyed by the instance's step count and row).
-// What bounds it: issue (D2Q16: 740 instructions per node and step in items of six
-// rows, 600 in long ones: at 2070 MHz 553k nodes cannot take less than 10.2 and
-// 8.2 us on 152 SMs) and the latency of each warp's chain, so it needs warps: the
+// What bounds it: issue (D2Q16: 651 thread-instructions per node and step in items
+// of five rows, 600 in long ones: at 2070 MHz 553k nodes cannot take less than 8.9
+// and 8.2 us on 152 SMs) and the latency of each warp's chain, so it needs warps: the
 // per-item coefficients and flags sit in shared memory (a dozen 16-byte reads per
 // row) instead of registers, which lets D2Q16 keep four blocks on an SM (165 ->
 // 128 registers) and D2Q36 run without spills (96 B before), on packed pairs.
@@ -1043,10 +1043,10 @@ cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s) {
 // the chip holds (by work: the classes run side by side), dealt to up to kChains
 // chains once they fill it.  A step's launch, first loads and last blocks cost
 // about 4 us whatever its size; beside three other chains that time is filled
-// (512 channels of 16 to 1024 rows, us per step with one chain at its best
-// rows -> four chains at the rule's: D2Q16 17.3 -> 13.8, D2Q36 47.4 -> 42.6,
-// D3Q64 31.9 -> 29.8).  Smaller batches keep one chain (32 channels: 3.3 us
-// against 3.6).  Rows stay while they are within a factor of two of the rule's
+// (512 channels of 16 to 1024 rows, us per step with one chain at its best rows
+// against four at the rule's, before a lane's coefficients waited for its rows:
+// D2Q16 17.3 and 13.8, D2Q36 47.4 and 42.6, D3Q64 31.9 and 29.8; now 13.2, 41.8
+// and 29.5).  Smaller batches keep one chain (32 channels: 3.3 us against 3.6).  Rows stay while they are within a factor of two of the rule's
 // and the step graph has room, so that admissions seldom rebuild it.
 void pick_rows(lesbgk_batch *b) {
   double work[kNumClasses] = {}, rows[kNumClasses] = {}, all = 0.0;

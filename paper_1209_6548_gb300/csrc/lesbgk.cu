@@ -1144,9 +1144,9 @@ __global__ void k_reduce_partials(const double *__restrict__ partial, int n, dou
 // swaps the buffers.
 // What bounds it: the latency of one node's chain, 0.7 us (D2Q16) or 1.7 us
 // (D2Q36), and 0.2 us for the cluster's barrier, while no scheduler has two
-// warps.  us per step over 512 steps, k_step -> this kernel: 4x64 D2Q16 2.70 ->
-// 0.94, D2Q36 4.1 -> 1.9, D3Q64 3.5 -> 1.5; 4x1000 D2Q16 3.0 -> 1.24; 32x64
-// D2Q16 2.7 -> 1.24; in a call of three steps 5.6 -> 4.2.
+// warps.  us per step over 512 steps, a launch per step -> this kernel: 4x64
+// D2Q16 2.41 -> 0.95, D2Q36 4.0 -> 1.9, D3Q64 3.2 -> 1.5; 4x1000 D2Q16 2.85 ->
+// 1.25; 32x64 D2Q16 2.42 -> 1.00; a call of three steps on 4x64 9.6 -> 5.4.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
