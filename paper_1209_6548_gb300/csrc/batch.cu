@@ -775,7 +775,8 @@ void with_class(int cls, Fn &&fn) {
 //     step on the four-block kernel, 21.9 on it).  By default rows, four-block
 //     kernel against it: 4 columns, 300 blocks 4.24 and 4.15, 400 in one chain
 //     4.40 and 5.02, 460 in four 5.08 and 4.64, 640 5.5 and 4.9, 1200 the same;
-//     16 columns, 400 blocks 4.31 and 3.86, 520 4.12 and 4.18, 640 4.3 and 5.1.
+//     8 to 32 columns, 220 to 290 blocks 3.0 to 3.3 and 3.7, 400 4.3 and 3.9,
+//     520 4.12 and 4.18, 640 4.3 and 5.1.
 //     Beside other classes only with rows of the caller's.
 //   drain: with the caller's rows, a lone chain of long items that leaves SMs
 //     part full starts each step after the previous one's end; blocks that
@@ -1086,7 +1087,7 @@ void pick_rows(lesbgk_batch *b) {
     StepChoice &c = b->choice_of[cls];
     const bool d2q16 = few_built(cls);
     c.few = d2q16 && (active == 1 || !b->auto_rows) &&
-            (b->W > 4 ? blocks < 0.8 * cap
+            (b->W > 4 ? blocks < 0.8 * cap && (!b->auto_rows || blocks >= 0.5 * cap)
                       : blocks < 0.5 * cap || (b->chains_of[cls] > 1 && blocks < 1.1 * cap));
     c.drain = !b->auto_rows && b->chains_of[cls] == 1 && r >= (d2q16 ? 8 : 4) && blocks > 0.55 * sms &&
               blocks <= 2.0 * sms;
