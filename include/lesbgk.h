@@ -370,7 +370,8 @@ int lesbgk_batch_set_rows(lesbgk_batch *b, int32_t rows, void *stream);
  * (steady walls) by one block for steps_per_launch time steps (an even divisor of 64; 0
  * keeps the current, 64 by default), reading and writing device memory once
  * per launch, while the other instances take one launch per step; in the
- * 64-step graphs the two run side by side.  A resident instance is one
+ * 64-step graphs the two run side by side (the steps of a call beyond a multiple
+ * of 64 take one launch each for all instances).  A resident instance is one
  * block's serial work, so tall ones are better left to the per-step kernel:
  * until this call (or lesbgk_batch_autotune), and again from
  * lesbgk_batch_set_auto, it is on where every solve of the batch is such an
@@ -382,7 +383,7 @@ int lesbgk_batch_get_launch(const lesbgk_batch *b, int32_t *rows, int32_t *resid
                             int32_t *resident_max_ny);
 /* The work list as it stands for one slot (any pointer may be NULL; rebuilds the
  * list on the stream where solves came or went): the rows of its step items (0:
- * the resident kernel holds it), the chains its class's solves are dealt to, and
+ * the resident kernel takes it, and single steps items of their own), the chains its class's solves are dealt to, and
  * the rows of the items by which residuals and moments read it (of several
  * items, the longest). */
 int lesbgk_batch_get_work(lesbgk_batch *b, int32_t slot, int32_t *step_rows, int32_t *chains, int32_t *read_rows,

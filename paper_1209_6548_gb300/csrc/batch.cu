@@ -805,7 +805,7 @@ struct lesbgk_batch {
   int capacity = 0, nx = 0, W = 0;
   InstDesc *d_desc = nullptr;
   WorkItem *d_items = nullptr;
-  int *d_range = nullptr;      // {first, count} per class of the items the per-step kernel takes, then per class and chain
+  int *d_range = nullptr;      // {first, count} per class of the items the per-step kernel takes, per class and chain, of resident solves
   int *d_range_all = nullptr;  // {first, count} per class of the items that cover every solve (residuals, moments)
   int *d_rlist = nullptr;      // resident instances, bucket after bucket
   int *d_rrange = nullptr;     // {first, count} per bucket
@@ -834,13 +834,14 @@ struct lesbgk_batch {
   int rows = 32;           // rows per work item where the caller sets them
   bool auto_rows = true;   // until then: rows and chains per class by pick_rows
   int rows_of[kNumClasses] = {}, chains_of[kNumClasses] = {};
-  StepChoice choice_of[kNumClasses] = {};
+  StepChoice choice_of[kNumClasses] = {}, choice_res = {};
   int par = 0;
   int sm_count = 0;
   LatTables lat[kNumClasses];
   bool lat_ready[kNumClasses] = {};
   cudaGraphExec_t graph = nullptr;
   int range_chain[kNumClasses][kChains][2] = {};
+  int range_res[2] = {};  // step items of the resident solves (single steps)
   int graph_grid[kNumClasses][kChains] = {};
   bool graph_dirty = true;
   std::unique_ptr<double[]> stage;  // fields on their way to the device (lesbgk_batch_add_many)
@@ -868,7 +869,7 @@ Layout0 fixed_layout(int capacity) {
   L.mass = o;  // per-item mass partial of the residual pass
   o = align_up(o + sizeof(double) * (size_t)capacity * kItemsPerSlot, 256);
   L.range = o;
-  o = align_up(o + sizeof(int) * 2 * kNumClasses * (1 + kChains), 256);
+  o = align_up(o + sizeof(int) * 2 * (kNumClasses * (1 + kChains) + 1), 256);
   L.range_all = o;
   o = align_up(o + sizeof(int) * 2 * kNumClasses, 256);
   L.rlist = o;
@@ -995,21 +996,6 @@ bool is_resident(const lesbgk_batch *b, const lesbgk_batch::Slot &sl) {
          sl.p.ny <= std::min(b->resident_ny, b->resident_limit);
 }
 
-// K steps of every resident instance: one launch per non-empty bucket.
-cudaError_t launch_resident(lesbgk_batch *b, int K, int p_in, int p_out, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  BatchArgs a = make_args(b, 0);
-  for (int k = 0; k < kBuckets && e == cudaSuccess; ++k) {
-    const int n = b->rrange[k][1];
-    if (!n) continue;
-    const int *rr = b->d_rrange + 2 * k;
-    const int *rl = b->d_rlist;
-    void *args[] = {&a, &rl, &rr, &K, &p_in, &p_out};
-    e = cudaLaunchKernel(resident_fn(b->W), dim3(n), dim3(kBBlock), args, resident_smem(b, k), s);
-  }
-  return e;
-}
-
 const int *chain_range(const lesbgk_batch *b, int cls, int chain) {
   return b->d_range + 2 * (kNumClasses + cls * kChains + chain);
 }
@@ -1021,14 +1007,16 @@ unsigned step_grid(const lesbgk_batch *b, int n_items) {
   return (unsigned)std::max<long long>(blocks, 1);
 }
 
-// One step of a class.
-cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s) {
+// One step of a range of a class's items.
+cudaError_t launch_items(lesbgk_batch *b, int cls, const int *d_range, int count, StepChoice choice, int par,
+                         cudaStream_t s) {
   BatchArgs a = make_args(b, cls);
-  const unsigned grid = step_grid(b, b->range[cls][1]);
+  a.range = d_range;
+  const unsigned grid = step_grid(b, count);
   void *args[] = {&a, &par};
   cudaLaunchAttribute at{};  // may be scheduled while the previous step runs (the kernel waits for it)
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = b->choice_of[cls].drain ? 0 : 1;
+  at.val.programmaticStreamSerializationAllowed = choice.drain ? 0 : 1;
   cudaLaunchConfig_t c{};
   c.gridDim = dim3(grid);
   c.blockDim = dim3(kBBlock);
@@ -1036,7 +1024,40 @@ cudaError_t launch_one_step(lesbgk_batch *b, int cls, int par, cudaStream_t s) {
   c.stream = s;
   c.attrs = &at;
   c.numAttrs = 1;
-  return cudaLaunchKernelExC(&c, step_kernel(cls, b->W, b->choice_of[cls].few), args);
+  return cudaLaunchKernelExC(&c, step_kernel(cls, b->W, choice.few), args);
+}
+
+// One step of every solve.  Resident solves step through their items here: a
+// launch of one step per bucket of them took 18 to 25 us (64 short channels; 3
+// now), most of it each block's load and store of its whole state.
+cudaError_t launch_one_step(lesbgk_batch *b, int par, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls)
+    if (b->range[cls][1])
+      e = launch_items(b, cls, b->d_range + 2 * cls, b->range[cls][1], b->choice_of[cls], par, s);
+  if (e == cudaSuccess && b->range_res[1])
+    e = launch_items(b, 0, b->d_range + 2 * kNumClasses * (1 + kChains), b->range_res[1], b->choice_res, par, s);
+  return e;
+}
+
+// Rows per item by which `rows` rows make one and a half times `cap` blocks.
+int rule_rows(const lesbgk_batch *b, double rows, double cap) {
+  return (int)std::fmax(1.0, std::fmin(64.0, std::ceil(rows / ((double)(kBBlock / b->W) * 1.5 * cap))));
+}
+
+// The launch choice for `rows` rows in items of r, with `cap` slots for blocks;
+// `lone`: beside no other class, `set`: at rows of the caller's.
+StepChoice choose_step(const lesbgk_batch *b, int cls, double rows, int r, int chains, double cap, bool lone, bool set) {
+  const double sms = b->sm_count > 0 ? b->sm_count : 152;
+  const double blocks = rows / ((double)(kBBlock / b->W) * r);
+  const bool d2q16 = few_built(cls);
+  StepChoice c{};
+  if (d2q16 && b->W <= 4)
+    c.few = (lone || set) && (blocks < 0.5 * cap || (chains > 1 && blocks < 1.1 * cap));
+  else if (d2q16)
+    c.few = blocks < 0.8 * cap && (set || (lone && blocks >= 0.5 * cap));
+  c.drain = set && chains == 1 && r >= (d2q16 ? 8 : 4) && blocks > 0.55 * sms && blocks <= 2.0 * sms;
+  return c;
 }
 
 // Rows per work item and chains of each class, from the solves it holds, until
@@ -1075,7 +1096,7 @@ void pick_rows(lesbgk_batch *b) {
     }
     const double cap = (cls % 3 == 0 ? 4 : 2) * sms * work[cls] / all;
     int r = b->rows;
-    if (b->auto_rows) r = (int)std::fmin(64.0, std::ceil(rows[cls] / (per_block * 1.5 * cap)));
+    if (b->auto_rows) r = rule_rows(b, rows[cls], cap);
     auto chains = [&](int at) { return rows[cls] / (per_block * at) > 0.75 * cap ? most : 1; };
     const int old = b->rows_of[cls];
     if (b->auto_rows && b->graph && old && 2 * old >= r && old <= 2 * r && b->chains_of[cls] == chains(old) &&
@@ -1083,14 +1104,7 @@ void pick_rows(lesbgk_batch *b) {
       continue;
     b->rows_of[cls] = r;
     b->chains_of[cls] = chains(r);
-    const double blocks = rows[cls] / (per_block * r);
-    StepChoice &c = b->choice_of[cls];
-    const bool d2q16 = few_built(cls);
-    c.few = d2q16 && (active == 1 || !b->auto_rows) &&
-            (b->W > 4 ? blocks < 0.8 * cap && (!b->auto_rows || blocks >= 0.5 * cap)
-                      : blocks < 0.5 * cap || (b->chains_of[cls] > 1 && blocks < 1.1 * cap));
-    c.drain = !b->auto_rows && b->chains_of[cls] == 1 && r >= (d2q16 ? 8 : 4) && blocks > 0.55 * sms &&
-              blocks <= 2.0 * sms;
+    b->choice_of[cls] = choose_step(b, cls, rows[cls], r, b->chains_of[cls], cap, active == 1, !b->auto_rows);
   }
 }
 
@@ -1157,6 +1171,23 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
     }
   }
   if (!own) b->read_items = b->items.size();
+  // The resident solves' items for single steps (at most 454 rows each, so half
+  // of a solve's room holds them beside those by which they are read).
+  double res_rows = 0.0;
+  for (const auto &sl : b->slots)
+    if (sl.used && is_resident(b, sl)) res_rows += sl.p.ny;
+  const double cap_res = 4.0 * (b->sm_count > 0 ? b->sm_count : 152);
+  const int r_res = rule_rows(b, res_rows, cap_res);
+  b->range_res[0] = (int)b->items.size();
+  for (int i = 0; i < b->capacity && res_rows > 0.0; ++i) {
+    const auto &sl = b->slots[i];
+    if (!sl.used || !is_resident(b, sl)) continue;
+    for (int y0 = 0; y0 < sl.p.ny; y0 += r_res) b->items.push_back({i, y0, std::min(r_res, sl.p.ny - y0), 0});
+  }
+  std::stable_sort(b->items.begin() + b->range_res[0], b->items.end(),
+                   [](const WorkItem &x, const WorkItem &y) { return x.rows > y.rows; });
+  b->range_res[1] = (int)b->items.size() - b->range_res[0];
+  b->choice_res = choose_step(b, 0, res_rows, r_res, 1, cap_res, true, false);
   if ((long long)b->items.size() > (long long)b->capacity * (long long)kItemsPerSlot)
     return fail(LESBGK_ESPACE, "work list of %zu items exceeds its room", b->items.size());
   std::vector<int> rlist;
@@ -1175,6 +1206,9 @@ int rebuild_items(lesbgk_batch *b, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_range, b->range, sizeof(b->range), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->d_range + 2 * kNumClasses, b->range_chain, sizeof(b->range_chain), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && b->range_res[1])
+    e = cudaMemcpyAsync(b->d_range + 2 * kNumClasses * (1 + kChains), b->range_res, sizeof(b->range_res),
+                        cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_range_all, b->range_all, sizeof(b->range_all), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && !rlist.empty())
     e = cudaMemcpyAsync(b->d_rlist, rlist.data(), sizeof(int) * rlist.size(), cudaMemcpyHostToDevice, s);
@@ -1346,7 +1380,7 @@ extern "C" int lesbgk_batch_create(int32_t capacity, int32_t nx, void *d_workspa
   for (int w : {1, 2, 4, 8, 16, 32})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(resident_fn(w), cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_range, 0, sizeof(int) * 2 * kNumClasses * (1 + kChains), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_range, 0, sizeof(int) * 2 * (kNumClasses * (1 + kChains) + 1), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_range_all, 0, sizeof(int) * 2 * kNumClasses, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_rrange, 0, sizeof(int) * 2 * kBuckets, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1642,9 +1676,7 @@ extern "C" int lesbgk_batch_step(lesbgk_batch *b, int64_t nsteps, void *stream) 
   if (int rc = ensure_items(b, s)) return rc;
   cudaError_t e = cudaSuccess;
   auto direct_step = [&]() {
-    for (int cls = 0; cls < kNumClasses && e == cudaSuccess; ++cls)
-      if (b->range[cls][1]) e = launch_one_step(b, cls, b->par, s);
-    if (e == cudaSuccess) e = launch_resident(b, 1, b->par, b->par ^ 1, s);
+    if (e == cudaSuccess) e = launch_one_step(b, b->par, s);
     if (e == cudaSuccess) {
       b->par ^= 1;  // the slots' current buffers are desc.f[par]
       for (auto &sl : b->slots)
